@@ -31,71 +31,34 @@
 
 using namespace frk;
 
-// Each call launches one sweep kernel for every class of a batch, its warps
-// shared among the classes by weighted blocks (warp_share.h); the weight
-// matters for the fingerprint (a bf16 weight of 100 or 150 instead of 125
-// leaves one class's warps finishing last).  Off: one launch per class.
-#ifndef FR_MIX_FP
-#define FR_MIX_FP 1
-#endif
-#ifndef FR_MIX_PACK
-#define FR_MIX_PACK 1
-#endif
-// Pack and unpack launches keep this percentage of each class's segments out
-// of the warps' own ranges and cut it into units of FR_UNIT_SEGS_PACK
-// segments, which warps claim at run time once their range is done (0: none;
-// the fingerprint keeps a static split).
-#ifndef FR_DYN_PCT_PACK
-#define FR_DYN_PCT_PACK 8
-#endif
-#ifndef FR_UNIT_SEGS_PACK
-#define FR_UNIT_SEGS_PACK 4
-#endif
-
-
 namespace {
 
-// One sweep class of one batch: its kernel specialization and its slices of
-// the decomposition's warp and chunk-list tables (a mixed decomposition has
-// one entry per batch covering all its classes).
-struct SweepClass {
-  uint32_t dtype = 0;
-  bool aligned = false;
-  uint64_t warp_off = 0;
-  uint64_t list_off = 0;
-  // mixed: per sweep class, its claimable units and where its chunk list starts
-  uint32_t unit_off[kClassCount] = {0, 0, 0, 0, 0, 0};
-  uint32_t n_units[kClassCount] = {0, 0, 0, 0, 0, 0};
-  uint32_t class_list[kClassCount] = {0, 0, 0, 0, 0, 0};
-};
-
+// One batch of a decomposition: its chunks, and its slices of the warp and
+// unit tables.
 struct BatchInfo {
   uint64_t c_begin = 0, c_end = 0;
-  std::vector<SweepClass> classes;
+  uint64_t warp_off = 0, unit_off = 0;
+  uint32_t n_units = 0;
+  bool any = false;  // some chunk has a body
 };
 
 // Per-warp work of every batch, with the chunk table that carries this
 // decomposition's block offsets and record ranges.
 struct Decomp {
-  bool mixed = false;  // one launch per batch for all its classes
   int n_ctas = 0;
-  uint32_t n_warps = 0;  // per class launch: n_ctas * warps per CTA
   std::vector<BatchInfo> batches;
   uint64_t n_recs = 0;
   ChunkDesc* d_chunks = nullptr;
-  WarpDesc* d_warps = nullptr;
-  uint32_t* d_lists = nullptr;
-  uint64_t* d_rec_nblk = nullptr;
+  PieceDesc* d_pieces = nullptr;
+  RunDesc* d_warps = nullptr;
   uint32_t* d_rec_mul = nullptr;  // per record: x^(8 * bytes after it in its chunk's body)
   Record* d_recs = nullptr;
-  WarpDesc* d_units = nullptr;  // mixed: claimable units of every batch
-  uint32_t* d_queue = nullptr;  // mixed: kQueueWords counters per batch (SweepParams::queue)
+  RunDesc* d_units = nullptr;  // claimable units of every batch
+  uint32_t* d_queue = nullptr;  // a claim counter per batch, kQueueWords apart (SweepParams::queue)
 };
 
-// Counters of one mixed launch: a claim count per class and a count of the
-// warps that have left (kernels.h, SweepParams::queue), padded to 32 bytes.
+// Claim counters lie in different 32-byte sectors.
 constexpr size_t kQueueWords = 8;
-static_assert(kQueueWords >= kClassCount + 1, "queue words");
 
 }  // namespace
 
@@ -215,8 +178,7 @@ cudaError_t upload(T** dst, const std::vector<T>& src) {
 void free_decomp(Decomp& D) {
   cudaFree(D.d_chunks);
   cudaFree(D.d_warps);
-  cudaFree(D.d_lists);
-  cudaFree(D.d_rec_nblk);
+  cudaFree(D.d_pieces);
   cudaFree(D.d_rec_mul);
   cudaFree(D.d_recs);
   cudaFree(D.d_units);
@@ -243,29 +205,20 @@ void free_device(fr_plan p) {
 // warp, and every (warp, chunk) overlap gets one record.  Records are numbered batch by batch, class
 // by class, so each chunk's records are consecutive.  `min_recs`: record slots
 // to allocate at least (list-mode calls use one slot per listed chunk).
-// Plain: every class gets all n_ctas * warps_per_cta warps (one launch per
-// class).  Mixed: the classes of a batch share them in proportion to their
-// weighted blocks, each class's warps spread round-robin over the CTAs.  For
-// pack and unpack (mix 2) the warps' ranges cover the first
-// (100 - FR_DYN_PCT_PACK)% of each class's segments and the rest becomes units
-// claimed at run time (their records follow the class's range records, in
-// block order).
+// The classes of a batch share the warps in proportion to their weighted
+// blocks (`share`: kShareFingerprint or kSharePack weights), each class's
+// warps spread round-robin over the CTAs.  For pack and unpack the warps'
+// runs cover most of each class's segments and the rest becomes units claimed
+// at run time (their pieces follow the class's own, in block order).
 cudaError_t build_decomp(const std::vector<ChunkDesc>& base, const std::vector<uint64_t>& bounds, int n_ctas,
-                         int warps_per_cta, int mix, uint64_t min_recs, Decomp& D) {
-  const bool mixed = mix != 0;  // 1: fingerprint weights, 2: pack / unpack weights
+                         int warps_per_cta, int share, uint64_t min_recs, Decomp& D) {
   const uint64_t W = static_cast<uint64_t>(n_ctas) * warps_per_cta;
-  D.mixed = mixed;
   D.n_ctas = n_ctas;
-  D.n_warps = static_cast<uint32_t>(W);
   std::vector<ChunkDesc> chunks = base;
-  std::vector<WarpDesc> warps;
-  std::vector<uint32_t> lists;
-  std::vector<uint64_t> rec_nblk;
+  std::vector<RunDesc> warps, units;
+  std::vector<PieceDesc> pieces;
   std::vector<uint32_t> rec_mul;
-  std::vector<WarpDesc> units;
-  const uint64_t unit_segs = FR_UNIT_SEGS_PACK;
-  const uint64_t dyn_pct = mix == kSharePack ? FR_DYN_PCT_PACK : 0;
-  const bool claims = mixed && dyn_pct > 0;
+  std::vector<uint32_t> lists;  // per class, its chunks with a body, in order
   for (ChunkDesc& d : chunks) {
     d.blk_begin = 0;
     d.first_rec = 0;
@@ -275,7 +228,7 @@ cudaError_t build_decomp(const std::vector<ChunkDesc>& base, const std::vector<u
     BatchInfo bi;
     bi.c_begin = bounds[b];
     bi.c_end = bounds[b + 1];
-    uint64_t class_blocks[6] = {0, 0, 0, 0, 0, 0};
+    uint64_t class_blocks[kClassCount] = {0, 0, 0, 0, 0, 0};
     for (uint64_t c = bi.c_begin; c < bi.c_end; ++c) {
       ChunkDesc& d = chunks[c];
       d.blk_begin = class_blocks[d.sweep_class];
@@ -290,7 +243,7 @@ cudaError_t build_decomp(const std::vector<ChunkDesc>& base, const std::vector<u
       std::vector<uint64_t> cost;  // cost[s]: estimated cost of segments [0, s)
     };
     std::vector<Cls> cl;
-    for (uint32_t cls = 0; cls < 6; ++cls) {
+    for (uint32_t cls = 0; cls < kClassCount; ++cls) {
       if (class_blocks[cls] == 0) continue;
       Cls q;
       q.cls = cls;
@@ -311,103 +264,83 @@ cudaError_t build_decomp(const std::vector<ChunkDesc>& base, const std::vector<u
       q.seg_start.push_back(class_blocks[cls]);
       cl.push_back(std::move(q));
     }
+    bi.warp_off = warps.size();
+    bi.unit_off = units.size();
     if (cl.empty()) {
       D.batches.push_back(bi);
       continue;
     }
-    // warps per class, and (mixed) slot[q * W + j] = the batch-warp index of
-    // class q's j-th warp
+    bi.any = true;
+    // warps per class; slot[q * W + j] = the batch-warp index of class q's j-th warp
     std::vector<uint64_t> wc(cl.size(), W);
-    std::vector<uint32_t> slot;
-    const uint64_t warp_base = warps.size();
-    if (mixed) {
-      double cost[6];
-      for (size_t q = 0; q < cl.size(); ++q)
-        cost[q] = static_cast<double>(class_blocks[cl[q].cls]) * block_weight(cl[q].cls / 2, mix);
-      share_warps(cost, static_cast<int>(cl.size()), W, wc.data());
-      slot.resize(cl.size() * W);
-      spread_warps(wc.data(), static_cast<int>(cl.size()), W, n_ctas, warps_per_cta, slot.data(), W);
-      warps.resize(warp_base + W);
-      SweepClass sc;
-      sc.warp_off = warp_base;
-      sc.list_off = 0;
-      bi.classes.push_back(sc);
-    }
+    std::vector<uint32_t> slot(cl.size() * W);
+    double cost[kClassCount];
+    for (size_t q = 0; q < cl.size(); ++q)
+      cost[q] = static_cast<double>(class_blocks[cl[q].cls]) * block_weight(cl[q].cls / 2, share);
+    share_warps(cost, static_cast<int>(cl.size()), W, wc.data());
+    spread_warps(wc.data(), static_cast<int>(cl.size()), W, n_ctas, warps_per_cta, slot.data(), W);
+    warps.resize(bi.warp_off + W);
     for (size_t q = 0; q < cl.size(); ++q) {
       const uint32_t cls = cl[q].cls;
       const size_t lbase = cl[q].list_off;
       const std::vector<uint64_t>& seg_start = cl[q].seg_start;
       const uint64_t n_seg = seg_start.size() - 1, Wq = wc[q];
-      const uint64_t n_fix = claims ? n_seg - n_seg * dyn_pct / 100 : n_seg;  // segments in the warps' ranges
-      SweepClass sc;
-      sc.dtype = cls / 2;
-      sc.aligned = (cls & 1u) != 0;
-      sc.warp_off = warps.size();
-      sc.list_off = lbase;
+      const uint64_t n_fix = n_seg - claimed_segs(n_seg, Wq, share);  // segments in the warps' ranges
       uint64_t k = 0;  // walks the class list monotonically
-      // the descriptor of class blocks [b0, b1), with one record per chunk it overlaps
+      // class blocks [b0, b1) as a run: one piece (and record) per chunk they overlap
       auto range = [&](uint64_t b0, uint64_t b1) {
-        WarpDesc wd;
-        std::memset(&wd, 0, sizeof wd);
-        wd.blk_begin = b0;
-        wd.nblk = b1 - b0;
-        wd.rec_base = static_cast<uint32_t>(rec_nblk.size());
-        wd.cls = cls;
-        wd.list_off = static_cast<uint32_t>(lbase);
-        if (b1 > b0) {
-          while (b0 >= chunks[lists[lbase + k]].blk_begin + chunks[lists[lbase + k]].len / kBlockBytes) ++k;
-          wd.first_chunk = static_cast<uint32_t>(k);
-          uint64_t bb = b0, j = k;
-          while (bb < b1) {
-            ChunkDesc& d = chunks[lists[lbase + j]];
-            const uint64_t end = d.blk_begin + d.len / kBlockBytes;
-            const uint64_t n = std::min(b1, end) - bb;
-            if (d.n_recs == 0) d.first_rec = static_cast<uint32_t>(rec_nblk.size());
-            d.n_recs += 1;
-            rec_nblk.push_back(n);
-            rec_mul.push_back(host_xpow8((end - bb - n) * kBlockBytes));
-            bb += n;
-            if (bb == end) ++j;
+        RunDesc rd;
+        rd.first = static_cast<uint32_t>(pieces.size());
+        rd.cls = cls;
+        rd.unused = 0;
+        while (b0 < b1) {
+          const uint32_t id = lists[lbase + k];
+          ChunkDesc& d = chunks[id];
+          const uint64_t off = b0 - d.blk_begin, nb = d.len / kBlockBytes;
+          if (off == nb) {
+            ++k;
+            continue;
           }
+          const uint64_t n = std::min(b1 - b0, nb - off);
+          if (d.n_recs == 0) d.first_rec = static_cast<uint32_t>(pieces.size());
+          d.n_recs += 1;
+          PieceDesc pd;
+          pd.addr = d.addr + off * kBlockBytes;
+          pd.payload_off = d.payload_off + off * kBlockBytes;
+          pd.seg = d.seg_base + static_cast<uint32_t>(off / kSegBlocks);
+          pd.nblk = static_cast<uint32_t>(n);
+          pd.chunk = id;
+          pd.unused = 0;
+          pieces.push_back(pd);
+          rec_mul.push_back(host_xpow8((nb - off - n) * kBlockBytes));
+          b0 += n;
         }
-        return wd;
+        rd.n = static_cast<uint32_t>(pieces.size()) - rd.first;
+        return rd;
       };
       // the warps' ranges: the first n_fix segments cut by estimated cost
       std::vector<uint64_t> bnd(Wq + 1);
       const std::vector<uint64_t>& cost = cl[q].cost;
       split_ranges([&](uint64_t i) { return cost[i]; }, n_fix, Wq, bnd.data());
-      for (uint64_t w = 0; w < Wq; ++w) {
-        const WarpDesc wd = range(seg_start[bnd[w]], seg_start[bnd[w + 1]]);
-        if (mixed)
-          warps[warp_base + slot[q * W + w]] = wd;
-        else
-          warps.push_back(wd);
-      }
-      if (mixed) {
-        SweepClass& ms = bi.classes.back();
-        ms.unit_off[cls] = static_cast<uint32_t>(units.size());
-        ms.class_list[cls] = static_cast<uint32_t>(lbase);
-        for (uint64_t u = n_fix; u < n_seg; u += unit_segs)
-          units.push_back(range(seg_start[u], seg_start[std::min(u + unit_segs, n_seg)]));
-        ms.n_units[cls] = static_cast<uint32_t>(units.size() - ms.unit_off[cls]);
-      } else {
-        bi.classes.push_back(sc);
+      for (uint64_t w = 0; w < Wq; ++w)
+        warps[bi.warp_off + slot[q * W + w]] = range(seg_start[bnd[w]], seg_start[bnd[w + 1]]);
+      for (uint64_t u = n_fix; u < n_seg;) {
+        const uint64_t n = unit_segs(n_seg - u, Wq);
+        units.push_back(range(seg_start[u], seg_start[u + n]));
+        u += n;
       }
     }
+    bi.n_units = static_cast<uint32_t>(units.size() - bi.unit_off);
     D.batches.push_back(bi);
   }
-  D.n_recs = rec_nblk.size();
+  D.n_recs = pieces.size();
   cudaError_t e = upload(&D.d_chunks, chunks);
   if (e == cudaSuccess) e = upload(&D.d_warps, warps);
-  if (e == cudaSuccess) e = upload(&D.d_lists, lists);
-  if (e == cudaSuccess) e = upload(&D.d_rec_nblk, rec_nblk);
+  if (e == cudaSuccess) e = upload(&D.d_pieces, pieces);
   if (e == cudaSuccess) e = upload(&D.d_rec_mul, rec_mul);
   if (e == cudaSuccess) e = upload(&D.d_units, units);
-  if (e == cudaSuccess && claims) {
-    const size_t qbytes = kQueueWords * sizeof(uint32_t) * std::max<size_t>(D.batches.size(), 1);
-    e = cudaMalloc(&D.d_queue, qbytes);
-    if (e == cudaSuccess) e = cudaMemset(D.d_queue, 0, qbytes);
-  }
+  if (e == cudaSuccess && !units.empty())
+    e = upload(&D.d_queue, std::vector<uint32_t>(kQueueWords * D.batches.size(), 0));
   const uint64_t slots = std::max<uint64_t>(D.n_recs, min_recs);
   if (e == cudaSuccess && slots) e = cudaMalloc(&D.d_recs, slots * sizeof(Record));
   return e;
@@ -417,44 +350,25 @@ cudaError_t build_decomp(const std::vector<ChunkDesc>& base, const std::vector<u
 fr_status run_batches(fr_plan p, const Decomp& D, int mode, uint8_t* packed, FpEntry* out_fp, size_t b0, size_t b1,
                       cudaStream_t s) {
   for (size_t b = b0; b < b1; ++b) {
-    for (const SweepClass& sc : D.batches[b].classes) {
-      SweepParams sp;
-      sp.chunks = D.d_chunks;
-      sp.warps = D.d_warps + sc.warp_off;
-      sp.class_chunks = D.d_lists;  // (WarpDesc::list_off is absolute)
-      sp.recs = D.d_recs;
-      sp.segs = p->d_segs;
-      sp.packed = packed;
-      sp.n_warps = D.n_warps;
-      sp.units = D.d_units;
-      sp.queue = D.d_queue ? D.d_queue + kQueueWords * b : nullptr;
-      for (uint32_t c = 0; c < kClassCount; ++c) {
-        sp.unit_off[c] = sc.unit_off[c];
-        sp.n_units[c] = sc.n_units[c];
-        sp.list_off[c] = sc.class_list[c];
-      }
-      cudaError_t e;
-      if (D.mixed)
-        e = mode == kModeFingerprint ? launch_sweep_fp_mixed(sp, D.n_ctas, s)
-            : mode == kModePack      ? launch_sweep_pack_mixed(sp, D.n_ctas, s)
-            : mode == kModeUnpackFp  ? launch_sweep_unpack_fp_mixed(sp, D.n_ctas, s)
-                                     : launch_sweep_unpack_mixed(sp, D.n_ctas, s);
-      else if (mode == kModeFingerprint)
-        e = launch_sweep_fp(sc.dtype, sc.aligned, sp, D.n_ctas, s);
-      else if (mode == kModePack)
-        e = launch_sweep_pack(sc.dtype, sc.aligned, sp, D.n_ctas, s);
-      else if (mode == kModeUnpackFp)
-        e = launch_sweep_unpack_fp(sc.dtype, sc.aligned, sp, D.n_ctas, s);
-      else
-        e = launch_sweep_unpack(sc.dtype, sc.aligned, sp, D.n_ctas, s);
-      if (e != cudaSuccess) return cuda_fail(e, "sweep kernel launch");
-    }
+    const BatchInfo& bi = D.batches[b];
+    if (!bi.any) continue;
+    SweepParams sp;
+    sp.pieces = D.d_pieces;
+    sp.warps = D.d_warps + bi.warp_off;
+    sp.recs = D.d_recs;
+    sp.segs = p->d_segs;
+    sp.packed = packed;
+    sp.units = D.d_units + bi.unit_off;
+    sp.queue = D.d_queue ? D.d_queue + kQueueWords * b : nullptr;
+    sp.n_units = bi.n_units;
+    const cudaError_t e = launch_sweep(mode, sp, D.n_ctas, s);
+    if (e != cudaSuccess) return cuda_fail(e, "sweep kernel launch");
   }
   FinalizeParams fp;
   fp.chunks = D.d_chunks;
   fp.recs = D.d_recs;
   fp.segs = p->d_segs;
-  fp.rec_nblk = D.d_rec_nblk;
+  fp.pieces = D.d_pieces;
   fp.rec_mul = D.d_rec_mul;
   fp.crc_xor = p->d_crc_xor;
   fp.n_chunks = p->n_chunks;
@@ -488,7 +402,7 @@ fr_status run_list(fr_plan p, int mode, const uint32_t* ids, uint64_t n, uint8_t
   fp.chunks = p->whole[0].d_chunks;
   fp.recs = p->whole[0].d_recs;
   fp.segs = p->d_segs;
-  fp.rec_nblk = nullptr;
+  fp.pieces = nullptr;
   fp.rec_mul = nullptr;
   fp.crc_xor = p->d_crc_xor;
   fp.n_chunks = p->n_chunks;
@@ -660,12 +574,11 @@ fr_status fr_plan_create_batched(const fr_tensor* tensors, uint64_t n_tensors, u
   // ---- decompositions
   e = cudaSuccess;
   if (n_chunks > 0) {
-    // distinct decompositions of the modes: warps per CTA and mixing (none,
-    // with the fingerprint's weights, with pack's); the fingerprint's is geo 0
-    std::vector<int> counts;  // 3 * warps + mix
+    // distinct decompositions of the modes: warps per CTA and class weights;
+    // the fingerprint's is geo 0
+    std::vector<int> counts;  // 3 * warps + weights
     for (int m = 0; m < 4; ++m) {
-      const int mix = m == kModeFingerprint ? (FR_MIX_FP ? 1 : 0) : (FR_MIX_PACK ? 2 : 0);
-      const int w = 3 * sweep_warps(m) + mix;
+      const int w = 3 * sweep_warps(m) + (m == kModeFingerprint ? kShareFingerprint : kSharePack);
       int g = 0;
       while (g < static_cast<int>(counts.size()) && counts[g] != w) ++g;
       if (g == static_cast<int>(counts.size())) counts.push_back(w);

@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(kFinThreads, FR_FIN_MINB) finalize_kernel(Fina
       uint64_t len = 0;
       if (have) {
         rec = p.recs[first_rec + i];
-        len = p.ids ? body : p.rec_nblk[first_rec + i] * kBlockBytes;
+        len = p.ids ? body : static_cast<uint64_t>(p.pieces[first_rec + i].nblk) * kBlockBytes;
       }
       uint64_t suf = len;  // bytes of this record and the later ones in the batch
 #pragma unroll

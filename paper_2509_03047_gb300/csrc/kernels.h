@@ -20,31 +20,24 @@ __host__ __device__ constexpr bool mode_unpacks(int m) { return m == kModeUnpack
 __host__ __device__ constexpr bool mode_sums(int m) { return m != kModeUnpack; }
 
 struct SweepParams {
-  const ChunkDesc* chunks;
-  const WarpDesc* warps;  // this class's per-warp ranges
-  const uint32_t* class_chunks;  // ids of this class's chunks with a body, in order
-  Record* recs;
+  const PieceDesc* pieces;
+  const RunDesc* warps;   // one run per warp of the launch, of any class
+  Record* recs;           // one per piece
   double* segs;           // segment sums of squares (all modes but kModeUnpack)
   uint8_t* packed;        // pack: destination; unpack: source; fingerprint: unused
-  uint32_t n_warps;       // warps with a descriptor
-  // Mixed launches: per sweep class c, n_units[c] work units at
-  // units + unit_off[c] (block order), claimed at run time by warps that have
-  // finished their own range, and list_off[c], where the class's chunk list
-  // starts.  queue[c] counts the claims on class c, queue[kClassCount] the
-  // warps that have left; all are zero when a launch starts and the last warp
-  // to leave puts them back to zero.  queue = null: no units.
-  const WarpDesc* units;
+  // Work units of any class, claimed one at a time by warps that have
+  // finished their own run.  *queue counts the claims: zero when a launch
+  // starts and again when it ends.  n_units = 0: no units, queue unused.
+  const RunDesc* units;
   uint32_t* queue;
-  uint32_t unit_off[kClassCount];
-  uint32_t n_units[kClassCount];
-  uint32_t list_off[kClassCount];
+  uint32_t n_units;
 };
 
 struct FinalizeParams {
   const ChunkDesc* chunks;
   const Record* recs;
   const double* segs;
-  const uint64_t* rec_nblk;
+  const PieceDesc* pieces;  // per record: its piece (read only without rec_mul)
   const uint32_t* rec_mul;  // per record: x^(8 * bytes after it in its chunk's body); null: computed here
   const uint32_t* crc_xor;  // per chunk: CRC preset/final-XOR term for its length; null: computed here
   uint64_t n_chunks;        // chunks of the whole plan
@@ -95,18 +88,18 @@ struct ListParams {
   uint8_t* packed;
 };
 
-// One class of chunks: element type and 16-byte alignment of its tensors.
-cudaError_t launch_sweep_fp(uint32_t dtype, bool aligned, const SweepParams& p, int n_ctas, cudaStream_t s);
-// Every class of a batch in one fingerprint launch (per-warp class in WarpDesc;
-// class_chunks = the whole chunk-list table).
-cudaError_t launch_sweep_fp_mixed(const SweepParams& p, int n_ctas, cudaStream_t s);
-cudaError_t launch_sweep_pack_mixed(const SweepParams& p, int n_ctas, cudaStream_t s);
-cudaError_t launch_sweep_unpack_mixed(const SweepParams& p, int n_ctas, cudaStream_t s);
-cudaError_t launch_sweep_unpack_fp_mixed(const SweepParams& p, int n_ctas, cudaStream_t s);
-cudaError_t launch_sweep_pack(uint32_t dtype, bool aligned, const SweepParams& p, int n_ctas, cudaStream_t s);
-cudaError_t launch_sweep_unpack(uint32_t dtype, bool aligned, const SweepParams& p, int n_ctas, cudaStream_t s);
+// Every class of a batch in one launch (per-run class in RunDesc).
+cudaError_t launch_sweep_fp(const SweepParams& p, int n_ctas, cudaStream_t s);
+cudaError_t launch_sweep_pack(const SweepParams& p, int n_ctas, cudaStream_t s);
+cudaError_t launch_sweep_unpack(const SweepParams& p, int n_ctas, cudaStream_t s);
+cudaError_t launch_sweep_unpack_fp(const SweepParams& p, int n_ctas, cudaStream_t s);
+inline cudaError_t launch_sweep(int mode, const SweepParams& p, int n_ctas, cudaStream_t s) {
+  return mode == kModeFingerprint ? launch_sweep_fp(p, n_ctas, s)
+         : mode == kModePack      ? launch_sweep_pack(p, n_ctas, s)
+         : mode == kModeUnpackFp  ? launch_sweep_unpack_fp(p, n_ctas, s)
+                                  : launch_sweep_unpack(p, n_ctas, s);
+}
 cudaError_t launch_list_pack(const ListParams& p, cudaStream_t s);
-cudaError_t launch_sweep_unpack_fp(uint32_t dtype, bool aligned, const SweepParams& p, int n_ctas, cudaStream_t s);
 cudaError_t launch_list_unpack(const ListParams& p, cudaStream_t s);
 cudaError_t launch_list_unpack_fp(const ListParams& p, cudaStream_t s);
 inline cudaError_t launch_list_sweep(int mode, const ListParams& p, cudaStream_t s) {

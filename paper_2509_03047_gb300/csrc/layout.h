@@ -9,8 +9,9 @@
 // warp the call's sweep launch gives that class (warp_share.h), so a class's
 // warps take about equal time whatever the tensor sizes.  A warp's range
 // overlaps
-// one or more chunks; each overlap is a "piece" and produces one record (raw
-// CRC, non-finite count).  Warp ranges start on segment boundaries.
+// one or more chunks; each overlap is a "piece" with a descriptor of its own
+// and produces one record (raw CRC, non-finite count).  Warp ranges start on
+// segment boundaries.
 // The records of a chunk are consecutive and in order.  The finalize kernel
 // (one warp per chunk) folds a chunk's records and its tail.
 #pragma once
@@ -61,7 +62,7 @@ struct ChunkDesc {       // 64 bytes
   uint64_t len;          // chunk bytes
   uint64_t tensor_off;   // offset of the chunk inside its tensor
   uint64_t payload_off;  // offset of the payload in the packed buffer
-  uint64_t blk_begin;    // first body block in its class's block stream
+  uint64_t blk_begin;    // first body block in its class's block stream (planning only)
   uint32_t tensor_idx;
   uint32_t dtype;
   uint32_t first_rec;    // records of this chunk: [first_rec, first_rec + n_recs)
@@ -71,15 +72,23 @@ struct ChunkDesc {       // 64 bytes
 };
 static_assert(sizeof(ChunkDesc) == 64, "ChunkDesc layout");
 
-struct WarpDesc {        // 32 bytes
-  uint64_t blk_begin;    // first block of this warp's range
-  uint64_t nblk;         // blocks in the range (0: idle warp)
-  uint32_t first_chunk;  // position, in the class's chunk list, of the chunk holding blk_begin
-  uint32_t rec_base;     // record index of the first piece
-  uint32_t cls;          // mixed launches: the sweep class of the warp's chunks
-  uint32_t list_off;     // mixed launches: where that class's chunk list starts
+struct PieceDesc {       // 32 bytes: consecutive blocks of one chunk, swept by one warp
+  uint64_t addr;         // device address of its first byte in the tensor
+  uint64_t payload_off;  // offset of that byte in the packed buffer
+  uint32_t seg;          // index of its first segment sum
+  uint32_t nblk;         // blocks
+  uint32_t chunk;
+  uint32_t unused;
 };
-static_assert(sizeof(WarpDesc) == 32, "WarpDesc layout");
+static_assert(sizeof(PieceDesc) == 32, "PieceDesc layout");
+
+struct RunDesc {         // 16 bytes: a run of pieces of one class
+  uint32_t first;        // index of the first piece
+  uint32_t n;            // pieces (0: nothing to do)
+  uint32_t cls;          // sweep class
+  uint32_t unused;
+};
+static_assert(sizeof(RunDesc) == 16, "RunDesc layout");
 
 struct Record {          // one piece's partial result
   uint32_t crc;          // raw CRC (preset 0, no final XOR) of the piece's bytes

@@ -45,10 +45,9 @@ constexpr uint64_t kMaxSegs = FR_STATIC_MAX_SEGMENTS;  // 16 KiB sum segments
 
 // Byte offsets of the tables inside the static array (256-byte aligned).
 constexpr uint64_t kOffChunks = 0;
-constexpr uint64_t kOffLists = align_up(kOffChunks + kMaxChunks * sizeof(ChunkDesc), 256);
-constexpr uint64_t kOffWarps = align_up(kOffLists + kMaxChunks * sizeof(uint32_t), 256);
-constexpr uint64_t kOffRecNblk = align_up(kOffWarps + kMaxWarps * sizeof(WarpDesc), 256);
-constexpr uint64_t kOffRecs = align_up(kOffRecNblk + kMaxRecs * sizeof(uint64_t), 256);
+constexpr uint64_t kOffWarps = align_up(kOffChunks + kMaxChunks * sizeof(ChunkDesc), 256);
+constexpr uint64_t kOffPieces = align_up(kOffWarps + kMaxWarps * sizeof(RunDesc), 256);
+constexpr uint64_t kOffRecs = align_up(kOffPieces + kMaxRecs * sizeof(PieceDesc), 256);
 constexpr uint64_t kOffSegs = align_up(kOffRecs + kMaxRecs * sizeof(Record), 256);
 constexpr uint64_t kScratchBytes = align_up(kOffSegs + kMaxSegs * sizeof(double), 256);
 static_assert(kScratchBytes < (8ull << 20), "the static scratch must stay modest");
@@ -61,9 +60,9 @@ static __device__ __align__(256) uint8_t g_static_scratch[kScratchBytes];
 // Host copies of the tables, staged here and copied into the scratch.
 struct HostTables {
   ChunkDesc chunks[kMaxChunks];
-  uint32_t lists[kMaxChunks];
-  WarpDesc warps[kMaxWarps];
-  uint64_t rec_nblk[kMaxRecs];
+  uint32_t lists[kMaxChunks];  // per class: its chunks with a body, in order
+  RunDesc warps[kMaxWarps];
+  PieceDesc pieces[kMaxRecs];
   uint64_t seg_start[kMaxSegs + 1];  // per class: block where each segment starts
   uint64_t seg_cost[kMaxSegs + 1];   // per class: estimated cost of its segments before each
   uint64_t bnd[kMaxWarps + 1];       // per class: the segment where each warp's range starts
@@ -215,63 +214,62 @@ extern "C" fr_status fr_fingerprint_static(const fr_tensor* tensors, uint64_t n_
     uint64_t k = 0;
     for (uint64_t w = 0; w < Wq; ++w) {
       const uint64_t b0 = h.seg_start[h.bnd[w]], b1 = h.seg_start[h.bnd[w + 1]];
-      WarpDesc& wd = h.warps[h.slot[q * kMaxWarps + w]];
-      std::memset(&wd, 0, sizeof wd);
-      wd.blk_begin = b0;
-      wd.nblk = b1 - b0;
-      wd.rec_base = static_cast<uint32_t>(n_recs);
-      wd.cls = cls;
-      wd.list_off = static_cast<uint32_t>(list_off);
-      if (b1 == b0) continue;
-      while (b0 >= h.chunks[list[k]].blk_begin + h.chunks[list[k]].len / kBlockBytes) ++k;
-      wd.first_chunk = static_cast<uint32_t>(k);
-      uint64_t b = b0, j = k;
-      while (b < b1) {
-        ChunkDesc& d = h.chunks[list[j]];
-        const uint64_t end = d.blk_begin + d.len / kBlockBytes;
-        const uint64_t n = std::min(b1, end) - b;
+      RunDesc& rd = h.warps[h.slot[q * kMaxWarps + w]];
+      rd.first = static_cast<uint32_t>(n_recs);
+      rd.cls = cls;
+      rd.unused = 0;
+      for (uint64_t b = b0; b < b1;) {
+        ChunkDesc& d = h.chunks[list[k]];
+        const uint64_t off = b - d.blk_begin, nb = d.len / kBlockBytes;
+        if (off == nb) {
+          ++k;
+          continue;
+        }
+        const uint64_t n = std::min(b1 - b, nb - off);
         if (d.n_recs == 0) d.first_rec = static_cast<uint32_t>(n_recs);
         d.n_recs += 1;
-        h.rec_nblk[n_recs++] = n;  // n_recs <= W + chunks <= kMaxRecs
+        PieceDesc& pd = h.pieces[n_recs++];  // n_recs <= W + chunks <= kMaxRecs
+        pd.addr = d.addr + off * kBlockBytes;
+        pd.payload_off = d.payload_off + off * kBlockBytes;
+        pd.seg = d.seg_base + static_cast<uint32_t>(off / kSegBlocks);
+        pd.nblk = static_cast<uint32_t>(n);
+        pd.chunk = list[k];
+        pd.unused = 0;
         b += n;
-        if (b == end) ++j;
       }
+      rd.n = static_cast<uint32_t>(n_recs) - rd.first;
     }
   }
   const uint64_t n_warps = n_cls > 0 ? W : 0;
 
   // ---- tables into the scratch, ordered on the caller's stream
   e = cudaMemcpyAsync(scratch + kOffChunks, h.chunks, n_chunks * sizeof(ChunkDesc), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && n_lists)
-    e = cudaMemcpyAsync(scratch + kOffLists, h.lists, n_lists * sizeof(uint32_t), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && n_warps)
-    e = cudaMemcpyAsync(scratch + kOffWarps, h.warps, n_warps * sizeof(WarpDesc), cudaMemcpyHostToDevice, s);
+    e = cudaMemcpyAsync(scratch + kOffWarps, h.warps, n_warps * sizeof(RunDesc), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && n_recs)
-    e = cudaMemcpyAsync(scratch + kOffRecNblk, h.rec_nblk, n_recs * sizeof(uint64_t), cudaMemcpyHostToDevice, s);
+    e = cudaMemcpyAsync(scratch + kOffPieces, h.pieces, n_recs * sizeof(PieceDesc), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return fail(e);
 
   const ChunkDesc* d_chunks = reinterpret_cast<const ChunkDesc*>(scratch + kOffChunks);
   Record* d_recs = reinterpret_cast<Record*>(scratch + kOffRecs);
   if (n_cls > 0) {
     SweepParams sp;
-    sp.chunks = d_chunks;
-    sp.warps = reinterpret_cast<const WarpDesc*>(scratch + kOffWarps);
-    sp.class_chunks = reinterpret_cast<const uint32_t*>(scratch + kOffLists);
+    sp.pieces = reinterpret_cast<const PieceDesc*>(scratch + kOffPieces);
+    sp.warps = reinterpret_cast<const RunDesc*>(scratch + kOffWarps);
     sp.recs = d_recs;
     sp.segs = reinterpret_cast<double*>(scratch + kOffSegs);
     sp.packed = nullptr;
-    sp.n_warps = static_cast<uint32_t>(W);
     sp.units = nullptr;  // the warps' ranges cover every block: no claimed units
     sp.queue = nullptr;
-    for (uint32_t c = 0; c < kClassCount; ++c) sp.unit_off[c] = sp.n_units[c] = sp.list_off[c] = 0;
-    e = launch_sweep_fp_mixed(sp, n_sm, s);
+    sp.n_units = 0;
+    e = launch_sweep_fp(sp, n_sm, s);
     if (e != cudaSuccess) return fail(e);
   }
   FinalizeParams fp;
   fp.chunks = d_chunks;
   fp.recs = d_recs;
   fp.segs = reinterpret_cast<const double*>(scratch + kOffSegs);
-  fp.rec_nblk = reinterpret_cast<const uint64_t*>(scratch + kOffRecNblk);
+  fp.pieces = reinterpret_cast<const PieceDesc*>(scratch + kOffPieces);
   fp.rec_mul = nullptr;  // shifts and CRC terms are computed in the finalize kernel
   fp.crc_xor = nullptr;
   fp.n_chunks = n_chunks;

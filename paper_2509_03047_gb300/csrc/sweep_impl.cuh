@@ -29,12 +29,10 @@
 // count per mode (the 128 KiB of lane-replicated tables fill most of shared
 // memory).  The plan sorts chunks into classes by element type and by whether
 // the tensor is 16-byte aligned; each class has its own block stream, cut
-// into per-warp ranges, and its own code specialization, so each warp runs a
-// single loop variant.  A call launches once for all its classes
-// (sweep_mixed_kernel: each warp dispatches on its range's class once);
-// pack and unpack warps then claim the last few percent of the work as small
-// units (see sweep_warp_claims).  sweep_{fp,pack,unpack,unpack_fp}.cu each
-// instantiate one mode.
+// into per-warp runs of pieces, and its own code specialization, so each warp
+// runs a single loop variant.  A call launches once for all its classes
+// (sweep_kernel); its warps then claim the last few percent of the work as
+// small units.  sweep_{fp,pack,unpack,unpack_fp}.cu each instantiate one mode.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -71,15 +69,6 @@ constexpr int kTableBytes = 4 * 256 * 32 * 4;  // 4 tables x 256 entries x 32 la
 #ifndef FR_STAGE_UNPACK
 #define FR_STAGE_UNPACK 4
 #endif
-#ifndef FR_AHEAD_FP
-#define FR_AHEAD_FP 1
-#endif
-#ifndef FR_AHEAD_PACK
-#define FR_AHEAD_PACK 0
-#endif
-#ifndef FR_AHEAD_UNPACK
-#define FR_AHEAD_UNPACK 0
-#endif
 #ifndef FR_LOADFIRST_FP
 #define FR_LOADFIRST_FP 0
 #endif
@@ -91,7 +80,7 @@ constexpr int kTableBytes = 4 * 256 * 32 * 4;  // 4 tables x 256 entries x 32 la
 #endif
 // Blocks per validity span: one sum segment (a power of two, a multiple of
 // every stage).
-constexpr int kSpan = static_cast<int>(kSegBlocks);
+constexpr uint32_t kSpan = static_cast<uint32_t>(kSegBlocks);
 
 typedef unsigned long long u64;
 
@@ -314,7 +303,7 @@ struct Exact {
   uint32_t nonfinite;
 };
 
-// Exact per-element fallback for this lane's units of blocks [b0, b1):
+// Exact per-element fallback for this lane's units of `n` blocks, the first at sp:
 // non-finite elements are counted; each finite square is added exactly --
 // for |x| in [2^-40, 2^56] as its fp32 product and FMA residual into an
 // unevaluated float pair by TwoSum, else (tiny or huge values, rare) in fp64,
@@ -326,12 +315,12 @@ struct Exact {
 // (Loading the units in register batches instead makes the compiler spill in
 // the hot loop that calls this.)
 template <int DT, int AL>
-__device__ __noinline__ Exact slow_span(const uint8_t* sp, uint64_t b0, uint64_t b1) {
-  for (uint64_t b = b0; b < b1; ++b) asm volatile("prefetch.global.L1 [%0];" ::"l"(sp + b * kBlockBytes));
+__device__ __noinline__ Exact slow_span(const uint8_t* sp, uint32_t n) {
+  for (uint32_t b = 0; b < n; ++b) asm volatile("prefetch.global.L1 [%0];" ::"l"(sp + b * kBlockBytes));
   float hi = 0.0f, lo = 0.0f;
   double d = 0.0;
   uint32_t nonfinite = 0;
-  for (uint64_t b = b0; b < b1; ++b) {
+  for (uint32_t b = 0; b < n; ++b) {
     const uint4 v = ld_unit<AL>(sp + b * kBlockBytes);
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -362,12 +351,12 @@ __device__ __noinline__ Exact slow_span(const uint8_t* sp, uint64_t b0, uint64_t
   return Exact{(static_cast<double>(hi) + static_cast<double>(lo)) + d, nonfinite};
 }
 
-// Whether this lane's units of blocks [b0, b1) hold only (signed) zeros.
+// Whether this lane's units of `n` blocks hold only (signed) zeros.
 template <int DT, int AL>
-__device__ __noinline__ bool span_is_zero(const uint8_t* sp, uint64_t b0, uint64_t b1) {
+__device__ __noinline__ bool span_is_zero(const uint8_t* sp, uint32_t n) {
   constexpr uint32_t kMask = (DT == kDtF32) ? 0x7FFFFFFFu : 0x7FFF7FFFu;
   uint32_t acc = 0;
-  for (uint64_t b = b0; b < b1; ++b) {
+  for (uint32_t b = 0; b < n; ++b) {
     const uint4 v = ld_unit<AL>(sp + b * kBlockBytes);
     acc |= (v.x | v.y | v.z | v.w) & kMask;
   }
@@ -405,16 +394,15 @@ __device__ __forceinline__ void prefetch_l2_lane0(const uint8_t* p, uint32_t byt
 }
 
 // Per-mode pipeline geometry: blocks per lane held in registers one stage
-// ahead, and spans (kSpan blocks) prefetched into L2 ahead of use.
-template <int MODE>
+// ahead, and whether the next span (kSpan blocks) is prefetched into L2.
 // Unpack with fingerprint values does pack's work per byte (copy, CRC, sums),
 // so it takes pack's geometry.
+template <int MODE>
 struct Geo {
   static constexpr bool kPackLike = MODE == kModePack || MODE == kModeUnpackFp;
   static constexpr int kStage = MODE == kModeFingerprint ? FR_STAGE_FP : (kPackLike ? FR_STAGE_PACK
                                                                                     : FR_STAGE_UNPACK);
-  static constexpr int kAhead = MODE == kModeFingerprint ? FR_AHEAD_FP : (kPackLike ? FR_AHEAD_PACK
-                                                                                    : FR_AHEAD_UNPACK);
+  static constexpr bool kPrefetch = MODE == kModeFingerprint;
   // Issue a unit's reload before consuming it (more load lead, one register
   // copy) or after (no copy): latency-bound modes want the former.
   static constexpr bool kLoadFirst = MODE == kModeFingerprint ? FR_LOADFIRST_FP
@@ -441,24 +429,24 @@ __device__ __forceinline__ void do_unit(Lane<MODE, DT>& L, const uint4& v, uint8
   if (kFp) fp_unit<DT>(v, L.f);
 }
 
-// End of a span [b0, b1) (one segment): the fast sums are kept if finite and
+// End of a span (one segment) of `n` blocks, the lane's first unit at sp: the fast sums are kept if finite and
 // either large enough that fp32 underflow is negligible (below 2^-77 relative)
 // or made of zeros only; otherwise the segment is summed exactly from a
 // reload.  The lanes' sums are then added in a fixed tree and lane 0 stores
 // the segment's sum (a float pair, see seg_value) at its index.
 template <int MODE, int DT, int SAL>
-__device__ __forceinline__ void span_end(Lane<MODE, DT>& L, const uint8_t* sp, uint64_t b0, uint64_t b1,
-                                         double* seg, uint32_t lane) {
+__device__ __forceinline__ void span_end(Lane<MODE, DT>& L, const uint8_t* sp, uint32_t n, double* seg,
+                                         uint32_t lane) {
   const u64 ab = add2(L.f.A, L.f.B);
   const float tot = lo_f(ab) + hi_f(ab);
   bool ok = tot < __int_as_float(0x7F800000);
-  if (ok && !(tot >= 0x1p-60f)) ok = span_is_zero<DT, SAL>(sp, b0, b1);
+  if (ok && !(tot >= 0x1p-60f)) ok = span_is_zero<DT, SAL>(sp, n);
   float hi = 0.0f, lo = 0.0f;
   double d = 0.0;
   if (ok) {
     fold_to_pair(L.f, hi, lo);
   } else {
-    const Exact x = slow_span<DT, SAL>(sp, b0, b1);
+    const Exact x = slow_span<DT, SAL>(sp, n);
     d = x.d;
     L.nonfinite += x.nonfinite;
   }
@@ -489,91 +477,44 @@ __device__ __forceinline__ void span_end(Lane<MODE, DT>& L, const uint8_t* sp, u
 // One piece: `nblk` 512-byte blocks from `src` (to `dst` for pack/unpack).
 // SAL / DAL: alignment class (16, 4 or 1 bytes) of the source / destination.
 //
-// Pipeline: lane 0 prefetches whole spans into L2 kAhead spans ahead with the
-// bulk-copy unit; each lane keeps kStage 16-byte units of the next stage in
+// Pipeline: for the fingerprint, lane 0 prefetches whole spans into L2 one span
+// ahead with the bulk-copy unit; each lane keeps kStage 16-byte units of the next stage in
 // flight in registers, which therefore mostly wait for L2.  Each span is one
 // sum segment: its fp32 sums start at zero, are checked at its end, and are
 // replaced by an exact sum from a reload when they fail.
 template <int MODE, int DT, int SAL, int DAL>
 __device__ __forceinline__ void sweep_piece(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst,
-                                            uint64_t nblk, uint32_t lane, Record* rec, double* segs) {
+                                            uint32_t nblk, uint32_t lane, Record* rec, double* seg) {
   constexpr bool kFp = mode_sums(MODE) && (DT != kDtBytes);
-  constexpr int kStage = Geo<MODE>::kStage;
-  constexpr int kAhead = Geo<MODE>::kAhead;
+  constexpr uint32_t kStage = Geo<MODE>::kStage;
+  constexpr bool kPrefetch = Geo<MODE>::kPrefetch && SAL == 16;
   constexpr uint32_t kStageBytes = kStage * kBlockBytes;
+  constexpr uint32_t kSpanBytes = kSpan * kBlockBytes;
   const uint32_t lb = lane << 2;
-  const uint8_t* sp = src + lane * 16;
-  uint8_t* wp = dst + lane * 16;
 
   // The first span goes to L2 now; each later one about a span before use.
-  if (kAhead > 0 && SAL == 16) {
-    const uint64_t n = nblk < kSpan ? nblk : kSpan;
-    prefetch_l2_lane0(src, static_cast<uint32_t>(n * kBlockBytes), lane);
-  }
+  if (kPrefetch) prefetch_l2_lane0(src, (nblk < kSpan ? nblk : kSpan) * kBlockBytes, lane);
 
   Lane<MODE, DT> L;
   L.s[0] = L.s[1] = L.s[2] = L.s[3] = 0;
   L.f = FpAcc{0ull, 0ull, 0ull, 0ull};
   L.nonfinite = 0;
 
+  // (Every unit is given a value here: a register that is only set under a
+  // condition is live, to the compiler, around every loop that encloses this
+  // one, through the code of every class -- 1,000 bytes of spills.)
   uint4 cur[kStage];
+  const uint8_t* lp = src + lane * 16;
+  uint8_t* wp = dst + lane * 16;
 #pragma unroll
-  for (int u = 0; u < kStage; ++u)
-    if (u < nblk) cur[u] = ld_unit<SAL>(sp + static_cast<uint64_t>(u) * kBlockBytes);
-  const uint8_t* lp = sp + kStageBytes;  // the next stage's loads
+  for (uint32_t u = 0; u < kStage; ++u)
+    cur[u] = u < nblk ? ld_unit<SAL>(lp + u * kBlockBytes) : make_uint4(0u, 0u, 0u, 0u);
+  lp += kStageBytes;  // the next stage's loads
 
-  // Three loops cover a piece: (1) whole spans whose following stage is
-  // whole too, each span (one sum segment) a call-free loop of kSpan/kStage
-  // stages with no branch, preceded by the L2 prefetch of the span kAhead
-  // ahead and followed by its validity check -- the bulk of a long piece;
-  // (2) the stages left whose following stage is still whole, one stage per
-  // iteration, a span's check and the next prefetch when a stage ends a span;
-  // (3) the last one or two stages, predicated.  Loop (2) keeps the
-  // predicated drain to under 2 * kStage blocks (it used to take the last
-  // span and a stage, and ran at half speed); loop (1) keeps long pieces on
-  // the tighter loop (with (2) alone the bf16 fingerprint lost 12% per warp).
-  uint64_t i = 0;  // first block of the current span
-  for (; i + kSpan + kStage <= nblk; i += kSpan) {
-    if (kAhead > 0 && SAL == 16 && lane == 0) {
-      const uint64_t pf = i + kSpan * kAhead;
-      if (pf < nblk) {
-        const uint64_t n = (nblk - pf < kSpan) ? nblk - pf : kSpan;
-        prefetch_l2(src + pf * kBlockBytes, static_cast<uint32_t>(n * kBlockBytes));
-      }
-    }
-#pragma unroll 1
-    for (int stg = 0; stg < kSpan / kStage; ++stg) {
+  // One stage whose following stage is whole.
+  auto stage = [&]() {
 #pragma unroll
-      for (int u = 0; u < kStage; ++u) {
-        if (Geo<MODE>::kLoadFirst) {
-          const uint4 v = cur[u];
-          cur[u] = ld_unit<SAL>(lp + u * kBlockBytes);
-          do_unit<MODE, DT, DAL>(L, v, wp + u * kBlockBytes, lb);
-        } else {
-          do_unit<MODE, DT, DAL>(L, cur[u], wp + u * kBlockBytes, lb);
-          cur[u] = ld_unit<SAL>(lp + u * kBlockBytes);
-        }
-      }
-      lp += kStageBytes;
-      wp += kStageBytes;
-    }
-    if (kFp) span_end<MODE, DT, SAL>(L, sp, i, i + kSpan, segs + i / kSpan, lane);
-  }
-  if (kAhead > 0 && SAL == 16) {  // loop (2) prefetches at span ends only
-    const uint64_t pf = i + kSpan * kAhead;
-    if (pf < nblk) {
-      const uint64_t n = (nblk - pf < kSpan) ? nblk - pf : kSpan;
-      prefetch_l2_lane0(src + pf * kBlockBytes, static_cast<uint32_t>(n * kBlockBytes), lane);
-    }
-  }
-  // Loop (2): stage j after i is steady if i + (j + 2) * kStage <= nblk.
-  uint32_t st = 0;  // stages of the current span done
-  const uint64_t left = nblk - i;
-  const uint32_t n_steady = left >= 2 * kStage ? static_cast<uint32_t>((left - kStage) / kStage) : 0u;
-#pragma unroll 1
-  for (uint32_t k = n_steady; k > 0; --k) {
-#pragma unroll
-    for (int u = 0; u < kStage; ++u) {
+    for (uint32_t u = 0; u < kStage; ++u) {
       if (Geo<MODE>::kLoadFirst) {
         const uint4 v = cur[u];
         cur[u] = ld_unit<SAL>(lp + u * kBlockBytes);
@@ -585,35 +526,51 @@ __device__ __forceinline__ void sweep_piece(const uint8_t* __restrict__ src, uin
     }
     lp += kStageBytes;
     wp += kStageBytes;
-    if (++st == kSpan / kStage) {
-      st = 0;
-      if (kFp) span_end<MODE, DT, SAL>(L, sp, i, i + kSpan, segs + i / kSpan, lane);
-      if (kAhead > 0 && SAL == 16) {
-        const uint64_t pf = i + kSpan + kSpan * kAhead;
-        if (pf < nblk) {
-          const uint64_t n = (nblk - pf < kSpan) ? nblk - pf : kSpan;
-          prefetch_l2_lane0(src + pf * kBlockBytes, static_cast<uint32_t>(n * kBlockBytes), lane);
-        }
-      }
-      i += kSpan;
+  };
+
+  // Three loops cover a piece: (1) whole spans whose following stage is
+  // whole too, each span (one sum segment) a call-free loop of kSpan/kStage
+  // stages with no branch, preceded by the L2 prefetch of the next span and
+  // followed by its validity check -- the bulk of a long piece; (2) the
+  // stages left whose following stage is still whole, fewer than a span; (3)
+  // the last one or two stages, predicated.  Loop (2) keeps the predicated
+  // drain, which runs at about half the rate, to under 2 * kStage blocks.
+  uint32_t left = nblk;  // blocks not swept yet
+  while (left >= kSpan + kStage) {
+    if (kPrefetch && lane == 0) {
+      const uint32_t n = left - kSpan < kSpan ? left - kSpan : kSpan;
+      prefetch_l2(lp - kStageBytes + kSpanBytes, n * kBlockBytes);
     }
+#pragma unroll 1
+    for (uint32_t st = 0; st < kSpan / kStage; ++st) stage();
+    if (kFp) span_end<MODE, DT, SAL>(L, lp - kSpanBytes - kStageBytes, kSpan, seg, lane);
+    ++seg;
+    left -= kSpan;
   }
-  i += static_cast<uint64_t>(st) * kStage;
-  // Drain: the last one or two stages (fewer than 2 * kStage blocks), with
-  // predicates.
-  for (; i < nblk; i += kStage) {
+  if (kPrefetch && left > kSpan)
+    prefetch_l2_lane0(lp - kStageBytes + kSpanBytes, (left - kSpan) * kBlockBytes, lane);
+  uint32_t done = 0;  // blocks of the current span swept, whole stages
+#pragma unroll 1
+  for (; left >= 2 * kStage; left -= kStage, done += kStage) stage();
+  while (left > 0) {
 #pragma unroll
-    for (int u = 0; u < kStage; ++u) {
-      if (i + u < nblk) {
+    for (uint32_t u = 0; u < kStage; ++u) {
+      if (u < left) {
         do_unit<MODE, DT, DAL>(L, cur[u], wp + u * kBlockBytes, lb);
-        if (i + kStage + u < nblk) cur[u] = ld_unit<SAL>(lp + u * kBlockBytes);
+        if (kStage + u < left) cur[u] = ld_unit<SAL>(lp + u * kBlockBytes);
       }
     }
     lp += kStageBytes;
     wp += kStageBytes;
-    const uint64_t end = (i + kStage < nblk) ? i + kStage : nblk;
-    if (kFp && ((end & (kSpan - 1)) == 0 || end == nblk))
-      span_end<MODE, DT, SAL>(L, sp, i & ~static_cast<uint64_t>(kSpan - 1), end, segs + i / kSpan, lane);
+    const uint32_t n = left < kStage ? left : kStage;
+    left -= n;
+    if (kFp && (left == 0 || done + n == kSpan)) {
+      span_end<MODE, DT, SAL>(L, lp - (done + 2 * kStage) * kBlockBytes, done + n, seg, lane);
+      ++seg;
+      done = 0;
+    } else {
+      done += n;
+    }
   }
 
   // ---- fold the 128 streams into the raw CRC of the piece
@@ -649,7 +606,7 @@ __device__ __forceinline__ void sweep_piece(const uint8_t* __restrict__ src, uin
 }
 
 template <int MODE, int DT, int AL>
-__device__ __forceinline__ void sweep_piece_al(const uint8_t* tensor, uint8_t* packed, uint64_t n,
+__device__ __forceinline__ void sweep_piece_al(const uint8_t* tensor, uint8_t* packed, uint32_t n,
                                                uint32_t lane, Record* rec, double* segs) {
   if (mode_unpacks(MODE))
     sweep_piece<MODE, DT, 16, AL>(packed, const_cast<uint8_t*>(tensor), n, lane, rec, segs);
@@ -657,160 +614,87 @@ __device__ __forceinline__ void sweep_piece_al(const uint8_t* tensor, uint8_t* p
     sweep_piece<MODE, DT, AL, 16>(tensor, packed, n, lane, rec, segs);
 }
 
-// Claims the next unit of class c for this warp: its index within the
-// class's units, or n_units[c] when none is left.
-__device__ __forceinline__ uint32_t claim_unit(const SweepParams& p, uint32_t c, uint32_t lane) {
-  uint32_t u = 0;
-  if (lane == 0) u = atomicAdd(p.queue + c, 1u);
-  return __shfl_sync(0xFFFFFFFFu, u, 0);
+// A run of consecutive pieces of one class: a warp's own range, or a unit it
+// claimed.  A piece's descriptor says all its sweep needs, so a piece costs
+// one dependent load before its data, and the next one's is already in L1.
+// ALIGNED: every chunk of the class is 16-byte aligned (128-bit loads and
+// stores); else the tensor side uses 32-bit or byte accesses, chosen per
+// piece.
+template <int MODE, int DT, bool ALIGNED>
+__device__ __forceinline__ void sweep_run(const SweepParams& p, uint32_t r, uint32_t n, uint32_t lane) {
+  for (; n > 0; --n, ++r) {
+    const PieceDesc d = p.pieces[r];
+    if (n > 1 && lane == 0) asm volatile("prefetch.global.L1 [%0];" ::"l"(p.pieces + r + 1));
+    const uint8_t* tensor = reinterpret_cast<const uint8_t*>(d.addr);
+    uint8_t* packed = (MODE == kModeFingerprint) ? nullptr : p.packed + d.payload_off;
+    double* segs = p.segs + d.seg;
+    if (ALIGNED) {
+      sweep_piece_al<MODE, DT, 16>(tensor, packed, d.nblk, lane, p.recs + r, segs);
+    } else if ((reinterpret_cast<uintptr_t>(tensor) & 3u) == 0) {
+      sweep_piece_al<MODE, DT, 4>(tensor, packed, d.nblk, lane, p.recs + r, segs);
+    } else {
+      sweep_piece_al<MODE, DT, 1>(tensor, packed, d.nblk, lane, p.recs + r, segs);
+    }
+  }
 }
 
-// Whether a mode's mixed launches take claimed units: pack and unpack, which
-// are bound by memory latency and whose warps' rates differ from SM to SM by
-// a few percent.  The issue-bound fingerprint keeps its static split: the
-// claim loop around its sweep costs it more registers than the tail it
-// would save.
+// One run by its class's code.  (Plain unpack only copies and checksums, so
+// it runs every element type as bytes.)
+template <int MODE>
+__device__ __forceinline__ void sweep_class(const SweepParams& p, const RunDesc& rd, uint32_t lane) {
+  if constexpr (!mode_sums(MODE)) {
+    if (rd.cls & 1u)
+      sweep_run<MODE, kDtBytes, true>(p, rd.first, rd.n, lane);
+    else
+      sweep_run<MODE, kDtBytes, false>(p, rd.first, rd.n, lane);
+  } else {
+    switch (rd.cls) {
+      case kDtF32 * 2 + 1: sweep_run<MODE, kDtF32, true>(p, rd.first, rd.n, lane); break;
+      case kDtBf16 * 2 + 1: sweep_run<MODE, kDtBf16, true>(p, rd.first, rd.n, lane); break;
+      case kDtBytes * 2 + 1: sweep_run<MODE, kDtBytes, true>(p, rd.first, rd.n, lane); break;
+      case kDtF32 * 2: sweep_run<MODE, kDtF32, false>(p, rd.first, rd.n, lane); break;
+      case kDtBf16 * 2: sweep_run<MODE, kDtBf16, false>(p, rd.first, rd.n, lane); break;
+      default: sweep_run<MODE, kDtBytes, false>(p, rd.first, rd.n, lane); break;
+    }
+  }
+}
+
+// Whether a mode's warps claim units: pack and unpack, which are bound by
+// memory latency and whose warps' rates differ from SM to SM by a few percent.
+// The fingerprint keeps a static split: it is bound by instruction issue, and
+// the start of each unit (claim, descriptors, first loads: about 4 us against
+// 10 us for its 32 KiB) costs its launch more than the tail (GPT-2 small: its
+// SMs end between 270 and 282 us without units, all at 295 with 8% in units).
 __host__ __device__ constexpr bool mode_claims(int m) { return m != kModeFingerprint; }
 
-// One warp's range of its class's block stream: the pieces it overlaps, in
-// order.  ALIGNED: every tensor of the class is 16-byte aligned (128-bit
-// loads and stores); else the tensor side uses 32-bit or byte accesses, chosen
-// per piece.
-template <int MODE, int DT, bool ALIGNED>
-__device__ __forceinline__ void sweep_warp(const SweepParams& p, const WarpDesc& wd, const uint32_t* class_chunks,
-                                           uint32_t lane) {
-  uint64_t b = wd.blk_begin, left = wd.nblk;
-  uint32_t k = wd.first_chunk, r = wd.rec_base;
-  while (left > 0) {
-    const ChunkDesc cd = p.chunks[class_chunks[k]];
-    const uint64_t nb = cd.len / kBlockBytes;
-    const uint64_t off = b - cd.blk_begin;
-    const uint64_t n = (left < nb - off) ? left : nb - off;
-    const uint8_t* tensor = reinterpret_cast<const uint8_t*>(cd.addr) + off * kBlockBytes;
-    uint8_t* packed = (MODE == kModeFingerprint) ? nullptr : p.packed + cd.payload_off + off * kBlockBytes;
-    double* segs = p.segs + cd.seg_base + off / kSegBlocks;
-    if (ALIGNED) {
-      sweep_piece_al<MODE, DT, 16>(tensor, packed, n, lane, p.recs + r, segs);
-    } else if ((reinterpret_cast<uintptr_t>(tensor) & 3u) == 0) {
-      sweep_piece_al<MODE, DT, 4>(tensor, packed, n, lane, p.recs + r, segs);
-    } else {
-      sweep_piece_al<MODE, DT, 1>(tensor, packed, n, lane, p.recs + r, segs);
-    }
-    ++r;
-    b += n;
-    left -= n;
-    ++k;
-  }
-}
-
-// One warp's range, then (pack and unpack launches with units, p.queue set)
-// the units of sweep class `cls` it claims, one at a time, until none is
-// left.  (Plain unpack runs every element type as bytes, so `cls` names the
-// class's queue, not the code.)
-template <int MODE, int DT, bool ALIGNED>
-__device__ __forceinline__ void sweep_warp_claims(const SweepParams& p, const WarpDesc& wd, uint32_t cls,
-                                                  uint32_t lane) {
-  const uint32_t* class_chunks = p.class_chunks + wd.list_off;
-  WarpDesc cur = wd;
-  for (;;) {
-    sweep_warp<MODE, DT, ALIGNED>(p, cur, class_chunks, lane);
-    if (p.queue == nullptr) return;
-    const uint32_t u = claim_unit(p, cls, lane);
-    if (u >= p.n_units[cls]) return;
-    cur = p.units[p.unit_off[cls] + u];
-  }
-}
-
-// One kernel per (mode, element type, alignment class).
-template <int MODE, int DT, bool ALIGNED>
+// Every class of a batch in one launch: each warp sweeps a run of its own
+// class, and the plan spreads each class's warps over all CTAs, so warps that
+// wait on memory and warps that are bound by instruction issue share every
+// SM.  For pack and unpack the runs cover most of each class's blocks; the
+// rest is cut into units that warps claim one at a time once their own run is
+// done, so the launch ends when the work does, not when its slowest warp
+// does.  Which warp sweeps a unit changes nothing in the results: a piece's
+// record and segment sums have fixed slots.
+//
+// The claim counter needs no reset: every warp claims until it is refused
+// once, so a launch makes exactly n_units + (its warps) claims, and atomicInc
+// wraps to zero on the last of them.  (A claim made before the sweep it
+// follows, to hide its round trip, holds a unit back from idle warps: GPT-2
+// small's unpack lost 4%.)
+template <int MODE>
 __global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) sweep_kernel(SweepParams p) {
   fill_tables<Cta<MODE>::kThreads>();
   __syncthreads();
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t w = blockIdx.x * Cta<MODE>::kWarps + (threadIdx.x >> 5);
-  if (w >= p.n_warps) return;
-  sweep_warp<MODE, DT, ALIGNED>(p, p.warps[w], p.class_chunks, lane);
-}
-
-// Class c's code for this mode: plain unpack only copies and checksums, so
-// it runs every element type as bytes.
-template <int MODE, uint32_t C>
-__device__ __forceinline__ void sweep_class(const SweepParams& p, const WarpDesc& wd, uint32_t lane) {
-  constexpr int DT = mode_sums(MODE) ? static_cast<int>(C / 2) : static_cast<int>(kDtBytes);
-  sweep_warp_claims<MODE, DT, (C & 1u) != 0>(p, wd, C, lane);
-}
-
-// Help with class c's units left once a warp's own class has none.
-template <int MODE, uint32_t C>
-__device__ __forceinline__ void help_class(const SweepParams& p, uint32_t lane) {
-  if (p.n_units[C] == 0) return;
-  WarpDesc none;
-  none.blk_begin = 0;
-  none.nblk = 0;
-  none.first_chunk = 0;
-  none.rec_base = 0;
-  none.cls = C;
-  none.list_off = p.list_off[C];
-  sweep_class<MODE, C>(p, none, lane);
-}
-
-// Every class of a batch in one launch: each warp sweeps a range of its own
-// class, and the plan spreads each class's warps over all CTAs, so warps that
-// wait on memory and warps that are bound by instruction issue share every
-// SM.  The ranges cover most of each class's blocks; the rest is cut into
-// small units that warps claim one at a time once their own range is done:
-// first their own class's, then, in a fixed order, every other class's, so
-// the launch ends when the work does, not when its slowest warp does.  Which
-// warp sweeps a unit changes nothing in the results: a unit's records and
-// segment sums have fixed slots.  (The class code is inlined once per call
-// site and no loop runs over classes: a loop around the inlined sweeps makes
-// the compiler keep every variant's registers live at once.)
-template <int MODE>
-__global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) sweep_mixed_kernel(SweepParams p) {
-  fill_tables<Cta<MODE>::kThreads>();
-  __syncthreads();
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t w = blockIdx.x * Cta<MODE>::kWarps + (threadIdx.x >> 5);
-  if constexpr (!mode_claims(MODE)) {
-    // the static split: each warp its own range, one dispatch on its class
-    if (w >= p.n_warps) return;
-    const WarpDesc wd = p.warps[w];
-    const uint32_t* list = p.class_chunks + wd.list_off;
-    switch (wd.cls) {
-      case kDtF32 * 2 + 1: sweep_warp<MODE, kDtF32, true>(p, wd, list, lane); break;
-      case kDtBf16 * 2 + 1: sweep_warp<MODE, kDtBf16, true>(p, wd, list, lane); break;
-      case kDtBytes * 2 + 1: sweep_warp<MODE, kDtBytes, true>(p, wd, list, lane); break;
-      case kDtF32 * 2: sweep_warp<MODE, kDtF32, false>(p, wd, list, lane); break;
-      case kDtBf16 * 2: sweep_warp<MODE, kDtBf16, false>(p, wd, list, lane); break;
-      default: sweep_warp<MODE, kDtBytes, false>(p, wd, list, lane); break;
-    }
-  } else {
-    if (w < p.n_warps) {
-      const WarpDesc wd = p.warps[w];
-      switch (wd.cls) {
-        case kDtF32 * 2 + 1: sweep_class<MODE, kDtF32 * 2 + 1>(p, wd, lane); break;
-        case kDtBf16 * 2 + 1: sweep_class<MODE, kDtBf16 * 2 + 1>(p, wd, lane); break;
-        case kDtBytes * 2 + 1: sweep_class<MODE, kDtBytes * 2 + 1>(p, wd, lane); break;
-        case kDtF32 * 2: sweep_class<MODE, kDtF32 * 2>(p, wd, lane); break;
-        case kDtBf16 * 2: sweep_class<MODE, kDtBf16 * 2>(p, wd, lane); break;
-        default: sweep_class<MODE, kDtBytes * 2>(p, wd, lane); break;
-      }
-    }
-    if (p.queue == nullptr) return;
-    help_class<MODE, kDtF32 * 2 + 1>(p, lane);
-    help_class<MODE, kDtBf16 * 2 + 1>(p, lane);
-    help_class<MODE, kDtBytes * 2 + 1>(p, lane);
-    help_class<MODE, kDtF32 * 2>(p, lane);
-    help_class<MODE, kDtBf16 * 2>(p, lane);
-    help_class<MODE, kDtBytes * 2>(p, lane);
-    // Every warp has made its last claim once it gets here; the last one out
-    // zeroes the queue for the next launch on this plan.
-    if (lane == 0) {
-      __threadfence();
-      if (atomicAdd(p.queue + kClassCount, 1u) == gridDim.x * Cta<MODE>::kWarps - 1) {
-        for (uint32_t c = 0; c <= kClassCount; ++c) atomicExch(p.queue + c, 0u);
-      }
-    }
+  RunDesc rd = p.warps[blockIdx.x * Cta<MODE>::kWarps + (threadIdx.x >> 5)];
+  for (;;) {
+    sweep_class<MODE>(p, rd, lane);
+    if (!mode_claims(MODE) || p.n_units == 0) return;
+    uint32_t u = 0;
+    if (lane == 0) u = atomicInc(p.queue, p.n_units + gridDim.x * Cta<MODE>::kWarps - 1);
+    u = __shfl_sync(0xFFFFFFFFu, u, 0);
+    if (u >= p.n_units) return;
+    rd = p.units[u];
   }
 }
 
@@ -818,7 +702,7 @@ __global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) sweep_mixed_kernel(Swe
 // ids[w] into recs[w].  Every variant is a separate function, so this cold
 // kernel's dispatch does not burden the registers of the hot ones.
 template <int MODE, int DT, bool ALIGNED>
-__device__ __noinline__ void list_piece(const uint8_t* tensor, uint8_t* packed, uint64_t n, uint32_t lane,
+__device__ __noinline__ void list_piece(const uint8_t* tensor, uint8_t* packed, uint32_t n, uint32_t lane,
                                         Record* rec, double* segs) {
   if (ALIGNED)
     sweep_piece_al<MODE, DT, 16>(tensor, packed, n, lane, rec, segs);
@@ -836,7 +720,7 @@ __global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) list_kernel(ListParams
   const uint64_t w = static_cast<uint64_t>(blockIdx.x) * Cta<MODE>::kWarps + (threadIdx.x >> 5);
   if (w >= p.n) return;
   const ChunkDesc cd = p.chunks[p.ids[w]];
-  const uint64_t nb = cd.len / kBlockBytes;
+  const uint32_t nb = static_cast<uint32_t>(cd.len / kBlockBytes);
   if (nb == 0) return;
   const uint8_t* tensor = reinterpret_cast<const uint8_t*>(cd.addr);
   uint8_t* packed = (MODE == kModeFingerprint) ? nullptr : p.packed + cd.payload_off;
@@ -864,54 +748,23 @@ cudaError_t launch_list(const ListParams& p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <int MODE, int DT, bool ALIGNED>
-cudaError_t configure_one() {
-  return cudaFuncSetAttribute(sweep_kernel<MODE, DT, ALIGNED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kTableBytes);
-}
-
-template <int MODE, int DT, bool ALIGNED>
-cudaError_t launch_one(const SweepParams& p, int n_ctas, cudaStream_t s) {
-  sweep_kernel<MODE, DT, ALIGNED><<<n_ctas, Cta<MODE>::kThreads, kTableBytes, s>>>(p);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
-// Configure / launch every class kernel of one mode (plain unpack ignores the
-// element type: it only checksums and copies).
+// Opt the kernels of one mode in to their shared-memory size; launch them.
 template <int MODE>
 cudaError_t configure_mode() {
-  cudaError_t e = cudaFuncSetAttribute(list_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
-  if (e == cudaSuccess) e = configure_one<MODE, kDtBytes, true>();
-  if (e == cudaSuccess) e = configure_one<MODE, kDtBytes, false>();
-  if (mode_sums(MODE)) {
-    if (e == cudaSuccess) e = configure_one<MODE, kDtBf16, true>();
-    if (e == cudaSuccess) e = configure_one<MODE, kDtBf16, false>();
-    if (e == cudaSuccess) e = configure_one<MODE, kDtF32, true>();
-    if (e == cudaSuccess) e = configure_one<MODE, kDtF32, false>();
+  cudaError_t e = cudaFuncSetAttribute(sweep_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
+  if constexpr (MODE != kModeFingerprint) {  // no call fingerprints a list
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(list_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
   }
   return e;
 }
 
 template <int MODE>
-cudaError_t configure_mixed() {
-  return cudaFuncSetAttribute(sweep_mixed_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
-}
-
-template <int MODE>
-cudaError_t launch_mixed(const SweepParams& p, int n_ctas, cudaStream_t s) {
-  sweep_mixed_kernel<MODE><<<n_ctas, Cta<MODE>::kThreads, kTableBytes, s>>>(p);
+cudaError_t launch_mode(const SweepParams& p, int n_ctas, cudaStream_t s) {
+  sweep_kernel<MODE><<<n_ctas, Cta<MODE>::kThreads, kTableBytes, s>>>(p);
   return cudaGetLastError();
-}
-
-template <int MODE>
-cudaError_t launch_mode(uint32_t dtype, bool aligned, const SweepParams& p, int n_ctas, cudaStream_t s) {
-  if (!mode_sums(MODE) || dtype == kDtBytes)
-    return aligned ? launch_one<MODE, kDtBytes, true>(p, n_ctas, s) : launch_one<MODE, kDtBytes, false>(p, n_ctas, s);
-  if (dtype == kDtBf16)
-    return aligned ? launch_one<MODE, kDtBf16, true>(p, n_ctas, s) : launch_one<MODE, kDtBf16, false>(p, n_ctas, s);
-  return aligned ? launch_one<MODE, kDtF32, true>(p, n_ctas, s) : launch_one<MODE, kDtF32, false>(p, n_ctas, s);
 }
 
 }  // namespace frk

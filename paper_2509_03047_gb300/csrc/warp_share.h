@@ -4,7 +4,7 @@
 //
 // A warp sweeps a range of one class only.  The classes are not equally
 // costly per block: a bf16 block holds twice the elements of an fp32 block,
-// so the fingerprint spends about a quarter more instructions on it, while
+// so the fingerprint spends about a third more instructions on it, while
 // pack and unpack are bound by memory in every class.  The warps are shared
 // in proportion to each class's blocks times its weight (percent of an fp32
 // block), so that the classes' warps finish together; each class's warps are
@@ -17,7 +17,10 @@
 #include "layout.h"
 
 #ifndef FR_MIX_W_BF16
-#define FR_MIX_W_BF16 125  // fingerprint: a bf16 block costs 1.25 fp32 blocks
+// Fingerprint: a bf16 block costs 1.35 fp32 blocks.  Measured, GPT-2 small
+// (1.7 GB) / Llama-8B shard (14 GB) in us: 1.25 306 / 2116, 1.30 309 / 2111,
+// 1.35 292 / 2116, 1.40 293 / 2127.
+#define FR_MIX_W_BF16 135
 #endif
 #ifndef FR_MIX_W_BF16_PACK
 #define FR_MIX_W_BF16_PACK 100  // pack and unpack: memory-bound, all blocks alike
@@ -42,6 +45,22 @@
 #endif
 #ifndef FR_SPLIT_PIECE
 #define FR_SPLIT_PIECE 16
+#endif
+
+// A pack or unpack launch keeps FR_DYN_PCT percent of each class's segments
+// out of the warps' own runs, as units of at most FR_UNIT_SEGS segments that
+// warps claim at run time, when the class has at least FR_CLAIM_MIN segments
+// per warp.  Measured on GB300, pack / unpack of GPT-2 small: no units 562 /
+// 564 us; 8% in units of 1, 2 and 4 segments 547 / 538, 545 / 538, 549 / 540;
+// 4% of 1 553 / 548.
+#ifndef FR_DYN_PCT
+#define FR_DYN_PCT 8
+#endif
+#ifndef FR_UNIT_SEGS
+#define FR_UNIT_SEGS 2
+#endif
+#ifndef FR_CLAIM_MIN
+#define FR_CLAIM_MIN 4
 #endif
 
 namespace frk {
@@ -105,6 +124,19 @@ inline void split_ranges(const Prefix& cost, uint64_t n, uint64_t Wq, uint64_t* 
     while (s < n && static_cast<unsigned __int128>(cost(s + 1)) * Wq <= target) ++s;
     bnd[w] = s;
   }
+}
+
+// How many of the last segments of a class of n, shared by Wq warps, are cut
+// into units (none for the fingerprint, see mode_claims, nor while the warps
+// have too few segments each for a tail to even out).
+inline uint64_t claimed_segs(uint64_t n, uint64_t Wq, int kind) {
+  return kind == kShareFingerprint || n < FR_CLAIM_MIN * Wq ? 0 : n * FR_DYN_PCT / 100;
+}
+// Segments of the unit cut where `left` remain: single ones at the end, so
+// that no warp starts a long unit when the others run out of work.
+inline uint64_t unit_segs(uint64_t left, uint64_t Wq) {
+  const uint64_t n = left > Wq ? FR_UNIT_SEGS : 1;
+  return n < left ? n : left;
 }
 
 // slot[q * stride + j] = launch-warp index of class q's j-th warp.  Slot i is

@@ -71,7 +71,7 @@ typedef enum {
 } fr_dtype;
 
 /* One tensor of the state: `nbytes` bytes of device memory at `ptr`
- * (any alignment; 16-byte-aligned tensors take the fast path).  nbytes must
+ * (any alignment; 16-byte-aligned tensors are the fastest).  nbytes must
  * be a multiple of the element size.  `flags` must be 0. */
 typedef struct {
   void* ptr;

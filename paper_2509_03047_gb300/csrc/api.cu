@@ -206,8 +206,8 @@ void free_device(fr_plan p) {
 // by class, so each chunk's records are consecutive.  `min_recs`: record slots
 // to allocate at least (list-mode calls use one slot per listed chunk).
 // The classes of a batch share the warps in proportion to their weighted
-// blocks (`share`: kShareFingerprint or kSharePack weights), each class's
-// warps spread round-robin over the CTAs.  For pack and unpack the warps'
+// blocks (`share`: kShareFingerprint or kSharePack weights), placed by
+// place_warps.  For pack and unpack the warps'
 // runs cover most of each class's segments and the rest becomes units claimed
 // at run time (their pieces follow the class's own, in block order).
 cudaError_t build_decomp(const std::vector<ChunkDesc>& base, const std::vector<uint64_t>& bounds, int n_ctas,
@@ -276,9 +276,11 @@ cudaError_t build_decomp(const std::vector<ChunkDesc>& base, const std::vector<u
     std::vector<uint32_t> slot(cl.size() * W);
     double cost[kClassCount];
     for (size_t q = 0; q < cl.size(); ++q)
-      cost[q] = static_cast<double>(class_blocks[cl[q].cls]) * block_weight(cl[q].cls / 2, share);
+      cost[q] = static_cast<double>(class_blocks[cl[q].cls]) * class_weight(cl[q].cls, share);
     share_warps(cost, static_cast<int>(cl.size()), W, wc.data());
-    spread_warps(wc.data(), static_cast<int>(cl.size()), W, n_ctas, warps_per_cta, slot.data(), W);
+    uint32_t cls_of[kClassCount];
+    for (size_t q = 0; q < cl.size(); ++q) cls_of[q] = cl[q].cls;
+    place_warps(cls_of, wc.data(), static_cast<int>(cl.size()), warps_per_cta, slot.data(), W);
     warps.resize(bi.warp_off + W);
     for (size_t q = 0; q < cl.size(); ++q) {
       const uint32_t cls = cl[q].cls;
@@ -548,8 +550,6 @@ fr_status fr_plan_create_batched(const fr_tensor* tensors, uint64_t n_tensors, u
   uint64_t payload = align_up(n_chunks * kHeaderBytes, kPayloadAlign);
   uint64_t c = 0;
   for (uint64_t t = 0; t < n_tensors; ++t) {
-    const bool aligned = (reinterpret_cast<uintptr_t>(tensors[t].ptr) % 16 == 0) && (chunk_bytes % 16 == 0);
-    const uint32_t cls = tensors[t].dtype * 2 + (aligned ? 1 : 0);
     for (uint64_t off = 0; off < tensors[t].nbytes; off += chunk_bytes) {
       ChunkDesc& d = p->chunks[c++];
       std::memset(&d, 0, sizeof d);
@@ -559,7 +559,7 @@ fr_status fr_plan_create_batched(const fr_tensor* tensors, uint64_t n_tensors, u
       d.payload_off = payload;
       d.tensor_idx = static_cast<uint32_t>(t);
       d.dtype = tensors[t].dtype;
-      d.sweep_class = cls;
+      d.sweep_class = d.dtype * 2 + (d.addr % 16 == 0 ? 1 : 0);
       d.seg_base = static_cast<uint32_t>(p->n_segs);
       p->n_segs += (d.len / kBlockBytes + kSegBlocks - 1) / kSegBlocks;
       payload += align_up(d.len, kPayloadAlign);

@@ -3,7 +3,7 @@
 // A plan splits every tensor into chunks (per tensor, chunk_bytes each, the
 // last one shorter).  Each chunk is a "body" of whole 512-byte blocks plus a
 // "tail" of len % 512 bytes.  Chunks fall into sweep classes by element type
-// and by whether their tensor is 16-byte aligned.  The bodies of a class's
+// and by whether they start on a 16-byte boundary.  The bodies of a class's
 // chunks, concatenated in chunk order, form one block stream that is cut into
 // ranges of equal estimated cost (bytes, segment ends, chunk starts), one per
 // warp the call's sweep launch gives that class (warp_share.h), so a class's
@@ -54,7 +54,7 @@ constexpr uint32_t kMagic = 0x31435246u;  // bytes 'F','R','C','1'
 constexpr uint32_t kVersion = 1;
 
 enum : uint32_t { kDtBytes = 0, kDtBf16 = 1, kDtF32 = 2 };
-// Sweep classes: element type * 2 + (tensor 16-byte aligned ? 1 : 0).
+// Sweep classes: element type * 2 + (chunk starts on a 16-byte boundary ? 1 : 0).
 constexpr uint32_t kClassCount = 6;
 
 struct ChunkDesc {       // 64 bytes
@@ -67,7 +67,7 @@ struct ChunkDesc {       // 64 bytes
   uint32_t dtype;
   uint32_t first_rec;    // records of this chunk: [first_rec, first_rec + n_recs)
   uint32_t n_recs;
-  uint32_t sweep_class;  // dtype * 2 + (tensor 16-byte aligned ? 1 : 0)
+  uint32_t sweep_class;  // dtype * 2 + (starts on a 16-byte boundary ? 1 : 0)
   uint32_t seg_base;     // index of the body's first segment sum
 };
 static_assert(sizeof(ChunkDesc) == 64, "ChunkDesc layout");

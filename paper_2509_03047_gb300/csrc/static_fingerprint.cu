@@ -153,8 +153,6 @@ extern "C" fr_status fr_fingerprint_static(const fr_tensor* tensors, uint64_t n_
   uint64_t class_blocks[kClasses] = {0, 0, 0, 0, 0, 0};
   uint64_t c = 0, seg = 0;
   for (uint64_t t = 0; t < n_tensors; ++t) {
-    const bool aligned = (reinterpret_cast<uintptr_t>(tensors[t].ptr) % 16 == 0) && (chunk_bytes % 16 == 0);
-    const uint32_t cls = tensors[t].dtype * 2 + (aligned ? 1 : 0);
     for (uint64_t off = 0; off < tensors[t].nbytes; off += chunk_bytes) {
       ChunkDesc& d = h.chunks[c++];
       std::memset(&d, 0, sizeof d);
@@ -162,14 +160,14 @@ extern "C" fr_status fr_fingerprint_static(const fr_tensor* tensors, uint64_t n_
       d.addr = reinterpret_cast<uint64_t>(tensors[t].ptr) + off;
       d.tensor_off = off;
       d.payload_off = payload;
-      d.blk_begin = class_blocks[cls];
-      d.tensor_idx = static_cast<uint32_t>(t);
+            d.tensor_idx = static_cast<uint32_t>(t);
       d.dtype = tensors[t].dtype;
-      d.sweep_class = cls;
+      d.sweep_class = d.dtype * 2 + (d.addr % 16 == 0 ? 1 : 0);
       d.seg_base = static_cast<uint32_t>(seg);
       seg += (d.len / kBlockBytes + kSegBlocks - 1) / kSegBlocks;
       payload += align_up(d.len, kPayloadAlign);
-      class_blocks[cls] += d.len / kBlockBytes;
+      d.blk_begin = class_blocks[d.sweep_class];
+      class_blocks[d.sweep_class] += d.len / kBlockBytes;
     }
   }
   // one launch for every class: the W warps shared by weighted blocks, each
@@ -181,12 +179,12 @@ extern "C" fr_status fr_fingerprint_static(const fr_tensor* tensors, uint64_t n_
   for (uint32_t cls = 0; cls < kClasses; ++cls) {
     if (class_blocks[cls] == 0) continue;
     cls_of[n_cls] = cls;
-    cost[n_cls] = static_cast<double>(class_blocks[cls]) * block_weight(cls / 2, kShareFingerprint);
+    cost[n_cls] = static_cast<double>(class_blocks[cls]) * class_weight(cls, kShareFingerprint);
     ++n_cls;
   }
   if (n_cls > 0) {
     share_warps(cost, n_cls, W, wc);
-    spread_warps(wc, n_cls, W, n_sm, sweep_warps(kModeFingerprint), h.slot, kMaxWarps);
+    place_warps(cls_of, wc, n_cls, sweep_warps(kModeFingerprint), h.slot, kMaxWarps);
   }
   uint64_t n_lists = 0, n_recs = 0;
   for (int q = 0; q < n_cls; ++q) {

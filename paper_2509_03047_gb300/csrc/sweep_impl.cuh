@@ -7,7 +7,8 @@
 // does the whole-512-byte-block part of every chunk in one HBM pass:
 //
 //  * copy engine: each lane moves 16 bytes per block with a coalesced 128-bit
-//    load and (pack/unpack) a coalesced 128-bit store;
+//    load and (pack/unpack) a coalesced 128-bit store, whatever the tensor's
+//    alignment (take16);
 //  * CRC-32C: the 128 words of a block are 128 interleaved CRC streams
 //    (lane l owns streams 4l..4l+3, four independent dependency chains), each
 //    advanced by s <- (s ^ w) * x^4096 with four byte lookups in tables kept in
@@ -28,7 +29,7 @@
 // No tensor cores: nothing here is a contraction.  One CTA per SM, with a warp
 // count per mode (the 128 KiB of lane-replicated tables fill most of shared
 // memory).  The plan sorts chunks into classes by element type and by whether
-// the tensor is 16-byte aligned; each class has its own block stream, cut
+// they start on a 16-byte boundary; each class has its own block stream, cut
 // into per-warp runs of pieces, and its own code specialization, so each warp
 // runs a single loop variant.  A call launches once for all its classes
 // (sweep_kernel); its warps then claim the last few percent of the work as
@@ -62,6 +63,12 @@ constexpr int kTableBytes = 4 * 256 * 32 * 4;  // 4 tables x 256 entries x 32 la
 // they rely on 4-block register stages and more warps (kernels.h).
 #ifndef FR_STAGE_FP
 #define FR_STAGE_FP 8
+#endif
+// The fingerprint of shifted chunks takes the shorter stage: its loop holds
+// the realignment too, and with 8-block stages the loops of two element types
+// outgrow the instruction cache (2.5 GB of views: 686 us, 597 with 4).
+#ifndef FR_STAGE_FP_SHIFT
+#define FR_STAGE_FP_SHIFT 4
 #endif
 #ifndef FR_STAGE_PACK
 #define FR_STAGE_PACK 4
@@ -163,11 +170,8 @@ __device__ __forceinline__ uint32_t mul_fold(int i, uint32_t a) {
 
 // ------------------------------------------------------------------ memory
 
-template <int AL>
-__device__ __forceinline__ uint4 ld_unit(const uint8_t* p);
-
-template <>
-__device__ __forceinline__ uint4 ld_unit<16>(const uint8_t* p) {
+// 16 bytes at p, a multiple of 16.
+__device__ __forceinline__ uint4 ld_unit(const uint8_t* p) {
   uint4 v;
   asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
       : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
@@ -175,48 +179,78 @@ __device__ __forceinline__ uint4 ld_unit<16>(const uint8_t* p) {
   return v;
 }
 
-template <>
-__device__ __forceinline__ uint4 ld_unit<4>(const uint8_t* p) {
-  const uint32_t* q = reinterpret_cast<const uint32_t*>(p);
-  return make_uint4(__ldg(q), __ldg(q + 1), __ldg(q + 2), __ldg(q + 3));
-}
-
-template <>
-__device__ __forceinline__ uint4 ld_unit<1>(const uint8_t* p) {
-  uint32_t w[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    w[j] = static_cast<uint32_t>(__ldg(p + 4 * j)) | (static_cast<uint32_t>(__ldg(p + 4 * j + 1)) << 8) |
-           (static_cast<uint32_t>(__ldg(p + 4 * j + 2)) << 16) |
-           (static_cast<uint32_t>(__ldg(p + 4 * j + 3)) << 24);
-  }
-  return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-template <int AL>
-__device__ __forceinline__ void st_unit(uint8_t* p, uint4 v);
-
-template <>
-__device__ __forceinline__ void st_unit<16>(uint8_t* p, uint4 v) {
+__device__ __forceinline__ void st_unit(uint8_t* p, const uint4& v) {
   asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z),
                "r"(v.w)
                : "memory");
 }
 
-template <>
-__device__ __forceinline__ void st_unit<4>(uint8_t* p, uint4 v) {
-  uint32_t* q = reinterpret_cast<uint32_t*>(p);
-  __stcs(q, v.x);
-  __stcs(q + 1, v.y);
-  __stcs(q + 2, v.z);
-  __stcs(q + 3, v.w);
+// Chunks that do not start on a 16-byte boundary move in 16-byte granules all
+// the same.  A lane's unit lies across two granules.  Reading, lane l loads
+// the one its unit ends in and gets the one it starts in from lane l - 1 by
+// shuffle (lane 0: from lane 31's of the block before); take16 cuts the unit
+// out.  Writing, lane l stores the granule its unit starts in, whose first
+// bytes are the end of lane l - 1's unit.  So every lane holds the same 16
+// bytes of the chunk as for an aligned chunk, and neither the CRC streams nor
+// the order of the sums change with the alignment.  A granule is only read if
+// it holds a byte of the piece, so no read reaches a page that the tensor does
+// not; its other bytes are dropped, and never written.
+//
+// Before, such chunks moved by 4-byte or single-byte accesses 16 bytes apart
+// from lane to lane: 4 or 16 times the load and store instructions, each
+// touching every line of the block.  GB300, 2.5 GB of views at any element
+// offset, us: fingerprint 1095 -> 597, pack 1025 -> 931, unpack 1495 -> 791.
+
+// 16 bytes from byte t on (0 <= t < 16, the same in every lane) of a then b.
+__device__ __forceinline__ uint4 take16(const uint4& a, const uint4& b, uint32_t t) {
+  uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x, w5 = b.y;
+  if (t & 8u) {
+    w0 = a.z;
+    w1 = a.w;
+    w2 = b.x;
+    w3 = b.y;
+    w4 = b.z;
+    w5 = b.w;
+  }
+  if (t & 4u) {
+    w0 = w1;
+    w1 = w2;
+    w2 = w3;
+    w3 = w4;
+    w4 = w5;
+  }
+  const uint32_t sh = 8u * (t & 3u);
+  return make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh), __funnelshift_r(w2, w3, sh),
+                    __funnelshift_r(w3, w4, sh));
 }
 
-template <>
-__device__ __forceinline__ void st_unit<1>(uint8_t* p, uint4 v) {
+// Lane `from`'s v.
+__device__ __forceinline__ uint4 shfl4(const uint4& v, uint32_t from) {
+  return make_uint4(__shfl_sync(0xFFFFFFFFu, v.x, from), __shfl_sync(0xFFFFFFFFu, v.y, from),
+                    __shfl_sync(0xFFFFFFFFu, v.z, from), __shfl_sync(0xFFFFFFFFu, v.w, from));
+}
+__device__ __forceinline__ uint4 select4(bool c, const uint4& a, const uint4& b) {
+  return make_uint4(c ? a.x : b.x, c ? a.y : b.y, c ? a.z : b.z, c ? a.w : b.w);
+}
+
+// The unit at p by itself; SHIFT: p need not be a multiple of 16.
+template <bool SHIFT>
+__device__ __forceinline__ uint4 ld_unit_at(const uint8_t* p) {
+  if (!SHIFT) return ld_unit(p);
+  const uint32_t t = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p)) & 15u;
+  const uint4 a = ld_unit(p - t);
+  return t ? take16(a, ld_unit(p - t + 16), t) : a;
+}
+
+// The bytes k of v with k < t (HEAD) or k >= t, as single stores from p on:
+// the first and the last granule of a piece whose destination is shifted
+// belong to it in part only.
+template <bool HEAD>
+__device__ __forceinline__ void st_part(uint8_t* p, const uint4& v, uint32_t t) {
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-  for (int j = 0; j < 16; ++j) p[j] = static_cast<uint8_t>(w[j >> 2] >> (8 * (j & 3)));
+  for (uint32_t k = 0; k < 16; ++k)
+    if (HEAD ? k < t : k >= t) p[HEAD ? k : k - t] = static_cast<uint8_t>(w[k >> 2] >> (8 * (k & 3)));
 }
 
 // ------------------------------------------------------------------ f32x2
@@ -314,14 +348,14 @@ struct Exact {
 // one, and the float pair keeps the arithmetic off GB300's narrow fp64 pipe.
 // (Loading the units in register batches instead makes the compiler spill in
 // the hot loop that calls this.)
-template <int DT, int AL>
+template <int DT, bool SHIFT>
 __device__ __noinline__ Exact slow_span(const uint8_t* sp, uint32_t n) {
   for (uint32_t b = 0; b < n; ++b) asm volatile("prefetch.global.L1 [%0];" ::"l"(sp + b * kBlockBytes));
   float hi = 0.0f, lo = 0.0f;
   double d = 0.0;
   uint32_t nonfinite = 0;
   for (uint32_t b = 0; b < n; ++b) {
-    const uint4 v = ld_unit<AL>(sp + b * kBlockBytes);
+    const uint4 v = ld_unit_at<SHIFT>(sp + b * kBlockBytes);
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -352,12 +386,12 @@ __device__ __noinline__ Exact slow_span(const uint8_t* sp, uint32_t n) {
 }
 
 // Whether this lane's units of `n` blocks hold only (signed) zeros.
-template <int DT, int AL>
+template <int DT, bool SHIFT>
 __device__ __noinline__ bool span_is_zero(const uint8_t* sp, uint32_t n) {
   constexpr uint32_t kMask = (DT == kDtF32) ? 0x7FFFFFFFu : 0x7FFF7FFFu;
   uint32_t acc = 0;
   for (uint32_t b = 0; b < n; ++b) {
-    const uint4 v = ld_unit<AL>(sp + b * kBlockBytes);
+    const uint4 v = ld_unit_at<SHIFT>(sp + b * kBlockBytes);
     acc |= (v.x | v.y | v.z | v.w) & kMask;
   }
   return acc == 0;
@@ -397,11 +431,11 @@ __device__ __forceinline__ void prefetch_l2_lane0(const uint8_t* p, uint32_t byt
 // ahead, and whether the next span (kSpan blocks) is prefetched into L2.
 // Unpack with fingerprint values does pack's work per byte (copy, CRC, sums),
 // so it takes pack's geometry.
-template <int MODE>
+template <int MODE, bool SHIFT>
 struct Geo {
   static constexpr bool kPackLike = MODE == kModePack || MODE == kModeUnpackFp;
-  static constexpr int kStage = MODE == kModeFingerprint ? FR_STAGE_FP : (kPackLike ? FR_STAGE_PACK
-                                                                                    : FR_STAGE_UNPACK);
+  static constexpr int kStage = MODE == kModeFingerprint ? (SHIFT ? FR_STAGE_FP_SHIFT : FR_STAGE_FP)
+                                                         : (kPackLike ? FR_STAGE_PACK : FR_STAGE_UNPACK);
   static constexpr bool kPrefetch = MODE == kModeFingerprint;
   // Issue a unit's reload before consuming it (more load lead, one register
   // copy) or after (no copy): latency-bound modes want the former.
@@ -416,12 +450,29 @@ struct Lane {
   uint32_t s[4];  // CRC streams 4l..4l+3
   FpAcc f;        // fp32 sums of the current span
   uint32_t nonfinite;
+  // shifted pieces only
+  uint32_t t;     // take16's t
+  uint4 carry;    // lane 0: lane 31's granule (source) or unit (destination) of the previous block
+  bool first;     // destination, lane 0: no block stored yet
 };
 
-template <int MODE, int DT, int DAL>
+template <int MODE, int DT, bool SHIFT>
 __device__ __forceinline__ void do_unit(Lane<MODE, DT>& L, const uint4& v, uint8_t* wp, uint32_t lb) {
   constexpr bool kFp = mode_sums(MODE) && (DT != kDtBytes);
-  if (MODE != kModeFingerprint) st_unit<DAL>(wp, v);
+  if (MODE != kModeFingerprint) {
+    if (SHIFT && mode_unpacks(MODE)) {
+      const uint4 y = shfl4(v, (lb / 4 + 31) & 31u);
+      const uint4 g = take16(select4(lb == 0, L.carry, y), v, L.t);
+      L.carry = y;
+      if (!L.first)
+        st_unit(wp, g);
+      else
+        st_part<true>(wp + 16 - L.t, v, L.t);
+      L.first = false;
+    } else {
+      st_unit(wp, v);
+    }
+  }
   L.s[0] = braid_step(L.s[0] ^ v.x, lb);
   L.s[1] = braid_step(L.s[1] ^ v.y, lb);
   L.s[2] = braid_step(L.s[2] ^ v.z, lb);
@@ -434,19 +485,19 @@ __device__ __forceinline__ void do_unit(Lane<MODE, DT>& L, const uint4& v, uint8
 // or made of zeros only; otherwise the segment is summed exactly from a
 // reload.  The lanes' sums are then added in a fixed tree and lane 0 stores
 // the segment's sum (a float pair, see seg_value) at its index.
-template <int MODE, int DT, int SAL>
+template <int MODE, int DT, bool SHIFT>
 __device__ __forceinline__ void span_end(Lane<MODE, DT>& L, const uint8_t* sp, uint32_t n, double* seg,
                                          uint32_t lane) {
   const u64 ab = add2(L.f.A, L.f.B);
   const float tot = lo_f(ab) + hi_f(ab);
   bool ok = tot < __int_as_float(0x7F800000);
-  if (ok && !(tot >= 0x1p-60f)) ok = span_is_zero<DT, SAL>(sp, n);
+  if (ok && !(tot >= 0x1p-60f)) ok = span_is_zero<DT, SHIFT>(sp, n);
   float hi = 0.0f, lo = 0.0f;
   double d = 0.0;
   if (ok) {
     fold_to_pair(L.f, hi, lo);
   } else {
-    const Exact x = slow_span<DT, SAL>(sp, n);
+    const Exact x = slow_span<DT, SHIFT>(sp, n);
     d = x.d;
     L.nonfinite += x.nonfinite;
   }
@@ -475,53 +526,77 @@ __device__ __forceinline__ void span_end(Lane<MODE, DT>& L, const uint8_t* sp, u
 }
 
 // One piece: `nblk` 512-byte blocks from `src` (to `dst` for pack/unpack).
-// SAL / DAL: alignment class (16, 4 or 1 bytes) of the source / destination.
+// SHIFT: the tensor side (source, or destination for unpack) does not start
+// on a 16-byte boundary; the packed side always does.
 //
 // Pipeline: for the fingerprint, lane 0 prefetches whole spans into L2 one span
 // ahead with the bulk-copy unit; each lane keeps kStage 16-byte units of the next stage in
 // flight in registers, which therefore mostly wait for L2.  Each span is one
 // sum segment: its fp32 sums start at zero, are checked at its end, and are
 // replaced by an exact sum from a reload when they fail.
-template <int MODE, int DT, int SAL, int DAL>
+template <int MODE, int DT, bool SHIFT>
 __device__ __forceinline__ void sweep_piece(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst,
                                             uint32_t nblk, uint32_t lane, Record* rec, double* seg) {
   constexpr bool kFp = mode_sums(MODE) && (DT != kDtBytes);
-  constexpr uint32_t kStage = Geo<MODE>::kStage;
-  constexpr bool kPrefetch = Geo<MODE>::kPrefetch && SAL == 16;
+  constexpr uint32_t kStage = Geo<MODE, SHIFT>::kStage;
+  constexpr bool kPrefetch = Geo<MODE, SHIFT>::kPrefetch;
+  constexpr bool kShiftSrc = SHIFT && !mode_unpacks(MODE), kShiftDst = SHIFT && mode_unpacks(MODE);
   constexpr uint32_t kStageBytes = kStage * kBlockBytes;
   constexpr uint32_t kSpanBytes = kSpan * kBlockBytes;
   const uint32_t lb = lane << 2;
-
-  // The first span goes to L2 now; each later one about a span before use.
-  if (kPrefetch) prefetch_l2_lane0(src, (nblk < kSpan ? nblk : kSpan) * kBlockBytes, lane);
 
   Lane<MODE, DT> L;
   L.s[0] = L.s[1] = L.s[2] = L.s[3] = 0;
   L.f = FpAcc{0ull, 0ull, 0ull, 0ull};
   L.nonfinite = 0;
+  const uint8_t* lp = src;
+  uint8_t* wp = dst;
+  if (kShiftSrc) {
+    L.t = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(src)) & 15u;
+    lp += 16u - L.t;
+    L.carry = lane == 0 ? ld_unit(lp - 16) : make_uint4(0u, 0u, 0u, 0u);
+  }
+  if (kShiftDst) {
+    const uint32_t before = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(dst)) & 15u;
+    L.t = 16u - before;
+    wp -= before;
+    L.carry = make_uint4(0u, 0u, 0u, 0u);
+    L.first = lane == 0;
+  }
+
+  // The first span goes to L2 now; each later one about a span before use.
+  if (kPrefetch) prefetch_l2_lane0(lp, (nblk < kSpan ? nblk : kSpan) * kBlockBytes, lane);
 
   // (Every unit is given a value here: a register that is only set under a
   // condition is live, to the compiler, around every loop that encloses this
   // one, through the code of every class -- 1,000 bytes of spills.)
   uint4 cur[kStage];
-  const uint8_t* lp = src + lane * 16;
-  uint8_t* wp = dst + lane * 16;
+  lp += lane * 16;
+  wp += lane * 16;
 #pragma unroll
   for (uint32_t u = 0; u < kStage; ++u)
-    cur[u] = u < nblk ? ld_unit<SAL>(lp + u * kBlockBytes) : make_uint4(0u, 0u, 0u, 0u);
+    cur[u] = u < nblk ? ld_unit(lp + u * kBlockBytes) : make_uint4(0u, 0u, 0u, 0u);
   lp += kStageBytes;  // the next stage's loads
 
+  // This lane's unit of the next block, which is in cur[u].
+  auto unit = [&](uint32_t u) {
+    if (!kShiftSrc) return cur[u];
+    const uint4 y = shfl4(cur[u], (lane + 31) & 31u);
+    const uint4 before = select4(lane == 0, L.carry, y);
+    L.carry = y;
+    return take16(before, cur[u], L.t);
+  };
   // One stage whose following stage is whole.
   auto stage = [&]() {
 #pragma unroll
     for (uint32_t u = 0; u < kStage; ++u) {
-      if (Geo<MODE>::kLoadFirst) {
-        const uint4 v = cur[u];
-        cur[u] = ld_unit<SAL>(lp + u * kBlockBytes);
-        do_unit<MODE, DT, DAL>(L, v, wp + u * kBlockBytes, lb);
+      if (Geo<MODE, SHIFT>::kLoadFirst) {
+        const uint4 v = unit(u);
+        cur[u] = ld_unit(lp + u * kBlockBytes);
+        do_unit<MODE, DT, SHIFT>(L, v, wp + u * kBlockBytes, lb);
       } else {
-        do_unit<MODE, DT, DAL>(L, cur[u], wp + u * kBlockBytes, lb);
-        cur[u] = ld_unit<SAL>(lp + u * kBlockBytes);
+        do_unit<MODE, DT, SHIFT>(L, unit(u), wp + u * kBlockBytes, lb);
+        cur[u] = ld_unit(lp + u * kBlockBytes);
       }
     }
     lp += kStageBytes;
@@ -543,7 +618,7 @@ __device__ __forceinline__ void sweep_piece(const uint8_t* __restrict__ src, uin
     }
 #pragma unroll 1
     for (uint32_t st = 0; st < kSpan / kStage; ++st) stage();
-    if (kFp) span_end<MODE, DT, SAL>(L, lp - kSpanBytes - kStageBytes, kSpan, seg, lane);
+    if (kFp) span_end<MODE, DT, kShiftSrc>(L, lp - kSpanBytes - kStageBytes - (kShiftSrc ? 16 - L.t : 0), kSpan, seg, lane);
     ++seg;
     left -= kSpan;
   }
@@ -556,8 +631,8 @@ __device__ __forceinline__ void sweep_piece(const uint8_t* __restrict__ src, uin
 #pragma unroll
     for (uint32_t u = 0; u < kStage; ++u) {
       if (u < left) {
-        do_unit<MODE, DT, DAL>(L, cur[u], wp + u * kBlockBytes, lb);
-        if (kStage + u < left) cur[u] = ld_unit<SAL>(lp + u * kBlockBytes);
+        do_unit<MODE, DT, SHIFT>(L, unit(u), wp + u * kBlockBytes, lb);
+        if (kStage + u < left) cur[u] = ld_unit(lp + u * kBlockBytes);
       }
     }
     lp += kStageBytes;
@@ -565,13 +640,17 @@ __device__ __forceinline__ void sweep_piece(const uint8_t* __restrict__ src, uin
     const uint32_t n = left < kStage ? left : kStage;
     left -= n;
     if (kFp && (left == 0 || done + n == kSpan)) {
-      span_end<MODE, DT, SAL>(L, lp - (done + 2 * kStage) * kBlockBytes, done + n, seg, lane);
+      span_end<MODE, DT, kShiftSrc>(L, lp - (done + 2 * kStage) * kBlockBytes - (kShiftSrc ? 16 - L.t : 0), done + n, seg,
+                                    lane);
       ++seg;
       done = 0;
     } else {
       done += n;
     }
   }
+
+  // A shifted destination ends in the first granule after the blocks.
+  if (kShiftDst && lane == 0) st_part<false>(dst - (16u - L.t) + static_cast<uint64_t>(nblk) * kBlockBytes, L.carry, L.t);
 
   // ---- fold the 128 streams into the raw CRC of the piece
   uint32_t v = mul_fold(0, L.s[0]) ^ L.s[1];
@@ -605,36 +684,20 @@ __device__ __forceinline__ void sweep_piece(const uint8_t* __restrict__ src, uin
   }
 }
 
-template <int MODE, int DT, int AL>
-__device__ __forceinline__ void sweep_piece_al(const uint8_t* tensor, uint8_t* packed, uint32_t n,
-                                               uint32_t lane, Record* rec, double* segs) {
-  if (mode_unpacks(MODE))
-    sweep_piece<MODE, DT, 16, AL>(packed, const_cast<uint8_t*>(tensor), n, lane, rec, segs);
-  else
-    sweep_piece<MODE, DT, AL, 16>(tensor, packed, n, lane, rec, segs);
-}
-
 // A run of consecutive pieces of one class: a warp's own range, or a unit it
 // claimed.  A piece's descriptor says all its sweep needs, so a piece costs
 // one dependent load before its data, and the next one's is already in L1.
-// ALIGNED: every chunk of the class is 16-byte aligned (128-bit loads and
-// stores); else the tensor side uses 32-bit or byte accesses, chosen per
-// piece.
+// ALIGNED: every chunk of the class starts on a 16-byte boundary of its
+// tensor's memory; else none does.
 template <int MODE, int DT, bool ALIGNED>
 __device__ __forceinline__ void sweep_run(const SweepParams& p, uint32_t r, uint32_t n, uint32_t lane) {
   for (; n > 0; --n, ++r) {
     const PieceDesc d = p.pieces[r];
     if (n > 1 && lane == 0) asm volatile("prefetch.global.L1 [%0];" ::"l"(p.pieces + r + 1));
-    const uint8_t* tensor = reinterpret_cast<const uint8_t*>(d.addr);
+    uint8_t* tensor = reinterpret_cast<uint8_t*>(d.addr);
     uint8_t* packed = (MODE == kModeFingerprint) ? nullptr : p.packed + d.payload_off;
-    double* segs = p.segs + d.seg;
-    if (ALIGNED) {
-      sweep_piece_al<MODE, DT, 16>(tensor, packed, d.nblk, lane, p.recs + r, segs);
-    } else if ((reinterpret_cast<uintptr_t>(tensor) & 3u) == 0) {
-      sweep_piece_al<MODE, DT, 4>(tensor, packed, d.nblk, lane, p.recs + r, segs);
-    } else {
-      sweep_piece_al<MODE, DT, 1>(tensor, packed, d.nblk, lane, p.recs + r, segs);
-    }
+    sweep_piece<MODE, DT, !ALIGNED>(mode_unpacks(MODE) ? packed : tensor, mode_unpacks(MODE) ? tensor : packed, d.nblk,
+                                    lane, p.recs + r, p.segs + d.seg);
   }
 }
 
@@ -702,14 +765,10 @@ __global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) sweep_kernel(SweepPara
 // ids[w] into recs[w].  Every variant is a separate function, so this cold
 // kernel's dispatch does not burden the registers of the hot ones.
 template <int MODE, int DT, bool ALIGNED>
-__device__ __noinline__ void list_piece(const uint8_t* tensor, uint8_t* packed, uint32_t n, uint32_t lane,
-                                        Record* rec, double* segs) {
-  if (ALIGNED)
-    sweep_piece_al<MODE, DT, 16>(tensor, packed, n, lane, rec, segs);
-  else if ((reinterpret_cast<uintptr_t>(tensor) & 3u) == 0)
-    sweep_piece_al<MODE, DT, 4>(tensor, packed, n, lane, rec, segs);
-  else
-    sweep_piece_al<MODE, DT, 1>(tensor, packed, n, lane, rec, segs);
+__device__ __noinline__ void list_piece(uint8_t* tensor, uint8_t* packed, uint32_t n, uint32_t lane, Record* rec,
+                                        double* segs) {
+  sweep_piece<MODE, DT, !ALIGNED>(mode_unpacks(MODE) ? packed : tensor, mode_unpacks(MODE) ? tensor : packed, n, lane,
+                                  rec, segs);
 }
 
 template <int MODE>
@@ -722,8 +781,8 @@ __global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) list_kernel(ListParams
   const ChunkDesc cd = p.chunks[p.ids[w]];
   const uint32_t nb = static_cast<uint32_t>(cd.len / kBlockBytes);
   if (nb == 0) return;
-  const uint8_t* tensor = reinterpret_cast<const uint8_t*>(cd.addr);
-  uint8_t* packed = (MODE == kModeFingerprint) ? nullptr : p.packed + cd.payload_off;
+  uint8_t* tensor = reinterpret_cast<uint8_t*>(cd.addr);
+  uint8_t* packed = p.packed + cd.payload_off;
   const bool aligned = (cd.sweep_class & 1u) != 0;
   const uint32_t dt = mode_sums(MODE) ? cd.dtype : kDtBytes;
   double* segs = p.segs + cd.seg_base;

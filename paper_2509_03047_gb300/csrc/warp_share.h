@@ -25,6 +25,12 @@
 #ifndef FR_MIX_W_BF16_PACK
 #define FR_MIX_W_BF16_PACK 100  // pack and unpack: memory-bound, all blocks alike
 #endif
+// Fingerprint: a block of a chunk off the 16-byte boundary costs 0.4 fp32
+// blocks more (0.2 / 0.4 / 0.6: 607 / 597 / 603 us for 2.5 GB of views); pack
+// and unpack even it out with their units.
+#ifndef FR_MIX_W_SHIFT
+#define FR_MIX_W_SHIFT 40
+#endif
 #ifndef FR_MIX_W_BYTES
 #define FR_MIX_W_BYTES 100
 #endif
@@ -72,6 +78,10 @@ inline double block_weight(uint32_t dt, int kind) {
   if (dt == kDtF32) return 100.0;
   if (dt == kDtBf16) return kind == kShareFingerprint ? FR_MIX_W_BF16 : FR_MIX_W_BF16_PACK;
   return FR_MIX_W_BYTES;
+}
+// Of sweep class `cls`.
+inline double class_weight(uint32_t cls, int kind) {
+  return block_weight(cls / 2, kind) + ((cls & 1u) == 0 && kind == kShareFingerprint ? FR_MIX_W_SHIFT : 0);
 }
 
 // wc[q] = warps of class q (q < n <= W): W shared in proportion to cost[q] > 0,
@@ -139,16 +149,54 @@ inline uint64_t unit_segs(uint64_t left, uint64_t Wq) {
   return n < left ? n : left;
 }
 
-// slot[q * stride + j] = launch-warp index of class q's j-th warp.  Slot i is
-// warp i / n_ctas of CTA i % n_ctas (round robin over the CTAs), and each
-// class takes a run of consecutive slots, so every CTA holds the floor or the
-// ceiling of its share of every class.  sum(wc) == W.
-inline void spread_warps(const uint64_t* wc, int n, uint64_t W, int n_ctas, int warps_per_cta, uint32_t* slot,
+// slot[q * stride + j] = launch-warp index of class q's j-th warp, for the m
+// classes q in `qs`, which share the launch warps [first, first + count); warp
+// w is warp w % warps_per_cta of CTA w / warps_per_cta.  The range's warps are
+// taken one per CTA in turn, and each class takes a run of consecutive ones,
+// so every whole CTA of the range holds the floor or the ceiling of its share
+// of every class.  The sum of wc[q] is count.
+inline void spread_range(const uint64_t* wc, const int* qs, int m, uint64_t first, uint64_t count, int warps_per_cta,
+                         uint32_t* slot, uint64_t stride) {
+  const uint64_t wpc = static_cast<uint64_t>(warps_per_cta), end = first + count;
+  uint64_t cta = first / wpc, row = 0;  // the next candidate: warp `row` of `cta`
+  for (int k = 0; k < m; ++k) {
+    for (uint64_t j = 0; j < wc[qs[k]];) {
+      const uint64_t w = cta * wpc + row;
+      if (w >= first && w < end) slot[static_cast<uint64_t>(qs[k]) * stride + j++] = static_cast<uint32_t>(w);
+      if (++cta * wpc >= end) cta = first / wpc, ++row;
+    }
+  }
+}
+
+// The same for n <= kClassCount classes over a whole launch of W warps.
+inline void spread_warps(const uint64_t* wc, int n, uint64_t W, int, int warps_per_cta, uint32_t* slot,
                          uint64_t stride) {
-  uint64_t i = 0;
-  for (int q = 0; q < n; ++q)
-    for (uint64_t j = 0; j < wc[q] && i < W; ++j, ++i)
-      slot[q * stride + j] = static_cast<uint32_t>((i % n_ctas) * warps_per_cta + i / n_ctas);
+  int qs[kClassCount];
+  for (int q = 0; q < n; ++q) qs[q] = q;
+  spread_range(wc, qs, n, 0, W, warps_per_cta, slot, stride);
+}
+
+// The warps of a launch's classes (class q is sweep class cls[q]): those of
+// shifted chunks on the first CTAs, those of aligned chunks on the others (one
+// CTA may hold both), each spread over its CTAs.  Element types share every
+// SM on purpose; but every class is a loop of its own, and four of them
+// outgrow an SM's instruction cache (2.5 GB of views, every class on every SM
+// / alignments apart: fingerprint 839 / 711 us with 37% of the instruction
+// fetches missing, pack 932 / 918).
+inline void place_warps(const uint32_t* cls, const uint64_t* wc, int n, int warps_per_cta, uint32_t* slot,
+                        uint64_t stride) {
+  uint64_t first = 0;
+  for (uint32_t aligned = 0; aligned < 2; ++aligned) {
+    int qs[kClassCount], m = 0;
+    uint64_t count = 0;
+    for (int q = 0; q < n; ++q)
+      if ((cls[q] & 1u) == aligned) {
+        qs[m++] = q;
+        count += wc[q];
+      }
+    spread_range(wc, qs, m, first, count, warps_per_cta, slot, stride);
+    first += count;
+  }
 }
 
 }  // namespace frk

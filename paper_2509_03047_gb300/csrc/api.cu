@@ -27,6 +27,7 @@
 #include "gf2.cuh"
 #include "kernels.h"
 #include "layout.h"
+#include "seg_walk.h"
 #include "warp_share.h"
 
 using namespace frk;
@@ -48,6 +49,7 @@ struct Decomp {
   int n_ctas = 0;
   std::vector<BatchInfo> batches;
   uint64_t n_recs = 0;
+  // in the plan's device memory
   ChunkDesc* d_chunks = nullptr;
   PieceDesc* d_pieces = nullptr;
   RunDesc* d_warps = nullptr;
@@ -64,6 +66,7 @@ constexpr size_t kQueueWords = 8;
 
 struct fr_plan_s {
   int device = 0;
+  void* d_memory = nullptr;  // everything below lives in this one allocation
   int n_sm = 0;
   uint64_t chunk_bytes = 0, n_chunks = 0, packed_bytes = 0, state_bytes = 0;
   uint32_t n_batches = 1;
@@ -166,186 +169,236 @@ struct DeviceGuard {
   }
 };
 
-template <class T>
-cudaError_t upload(T** dst, const std::vector<T>& src) {
-  *dst = nullptr;
-  if (src.empty()) return cudaSuccess;
-  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(dst), src.size() * sizeof(T));
-  if (e != cudaSuccess) return e;
-  return cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
-}
+// A plan's device memory: tables gathered on the host, then scratch, as one
+// allocation and one copy.  (An allocation and a copy for each table, 40 of both
+// for a batched plan, were half of the 2.6 ms that a plan over 8 tensors in 8
+// batches took; it takes 0.6 ms now.)
+class PlanMemory {
+ public:
+  template <class T>
+  void table(T** at, const std::vector<T>& src) {
+    if (src.empty()) return;
+    const uint64_t off = align_up(tables_.size(), kAlign);
+    tables_.resize(off + src.size() * sizeof(T));
+    std::memcpy(tables_.data() + off, src.data(), src.size() * sizeof(T));
+    places_.push_back({reinterpret_cast<void**>(at), off, false});
+  }
+  template <class T>
+  void scratch(T** at, uint64_t count) {
+    if (count == 0) return;
+    places_.push_back({reinterpret_cast<void**>(at), scratch_, true});
+    scratch_ = align_up(scratch_ + count * sizeof(T), kAlign);
+  }
+  // Allocates, copies the tables and sets every pointer.
+  cudaError_t commit(void** memory) {
+    const uint64_t first = align_up(tables_.size(), kAlign);
+    cudaError_t e = cudaMalloc(memory, std::max<uint64_t>(first + scratch_, kAlign));
+    if (e != cudaSuccess) return e;
+    if (!tables_.empty()) e = cudaMemcpy(*memory, tables_.data(), tables_.size(), cudaMemcpyHostToDevice);
+    for (const Place& q : places_) *q.at = static_cast<uint8_t*>(*memory) + (q.scratch ? first : 0) + q.off;
+    return e;
+  }
 
-void free_decomp(Decomp& D) {
-  cudaFree(D.d_chunks);
-  cudaFree(D.d_warps);
-  cudaFree(D.d_pieces);
-  cudaFree(D.d_rec_mul);
-  cudaFree(D.d_recs);
-  cudaFree(D.d_units);
-  cudaFree(D.d_queue);
-  D = Decomp();
-}
+ private:
+  static constexpr uint64_t kAlign = 256;
+  struct Place {
+    void** at;
+    uint64_t off;
+    bool scratch;
+  };
+  std::vector<uint8_t> tables_;
+  std::vector<Place> places_;
+  uint64_t scratch_ = 0;
+};
 
 void free_device(fr_plan p) {
-  for (Decomp& d : p->whole) free_decomp(d);
-  for (Decomp& d : p->batched) free_decomp(d);
-  cudaFree(p->d_segs);
-  cudaFree(p->d_crc_xor);
-  cudaFree(p->d_flags);
-  cudaFree(p->d_status);
-  cudaFree(p->d_ids);
-  cudaFree(p->d_count);
+  cudaFree(p->d_memory);
   for (cudaEvent_t ev : p->events) cudaEventDestroy(ev);
   p->events.clear();
 }
 
 // Cut the chunks [bounds[b], bounds[b+1]) of every batch b into sweep work for
 // `n_ctas` CTAs: per batch and class, the class's 16 KiB segments in chunk
-// order are split into runs of equal estimated cost (split_ranges), one per
-// warp, and every (warp, chunk) overlap gets one record.  Records are numbered batch by batch, class
-// by class, so each chunk's records are consecutive.  `min_recs`: record slots
-// to allocate at least (list-mode calls use one slot per listed chunk).
+// order are split into runs of equal estimated cost (the rule of
+// split_ranges), one per warp, and every (warp, chunk) overlap is a piece with
+// a record.  Records are numbered batch by batch, class by class, so each
+// chunk's records are consecutive.  `min_recs`: record slots to allocate at
+// least (list-mode calls use one slot per listed chunk).
 // The classes of a batch share the warps in proportion to their weighted
 // blocks (`share`: kShareFingerprint or kSharePack weights), placed by
-// place_warps.  For pack and unpack the warps'
-// runs cover most of each class's segments and the rest becomes units claimed
-// at run time (their pieces follow the class's own, in block order).
-cudaError_t build_decomp(const std::vector<ChunkDesc>& base, const std::vector<uint64_t>& bounds, int n_ctas,
-                         int warps_per_cta, int share, uint64_t min_recs, Decomp& D) {
+// place_warps.  For pack and unpack the warps' runs cover most of each class's
+// segments and the rest becomes units claimed at run time (their pieces follow
+// the class's own, in block order).
+void build_decomp(const std::vector<ChunkDesc>& base, const std::vector<uint64_t>& bounds, int n_ctas,
+                  int warps_per_cta, int share, uint64_t min_recs, Decomp& D, PlanMemory& mem) {
   const uint64_t W = static_cast<uint64_t>(n_ctas) * warps_per_cta;
   D.n_ctas = n_ctas;
   std::vector<ChunkDesc> chunks = base;
   std::vector<RunDesc> warps, units;
   std::vector<PieceDesc> pieces;
   std::vector<uint32_t> rec_mul;
-  std::vector<uint32_t> lists;  // per class, its chunks with a body, in order
-  for (ChunkDesc& d : chunks) {
-    d.blk_begin = 0;
-    d.first_rec = 0;
-    d.n_recs = 0;
-  }
+  std::vector<uint32_t> lists[kClassCount];  // per class, the batch's chunks with a body, in order
+  std::vector<uint32_t> slot(kClassCount * W);
+  auto add_piece = [&](const PieceDesc& pd, uint64_t blocks_after) {
+    pieces.push_back(pd);
+    rec_mul.push_back(host_xpow8_blocks(blocks_after));
+  };
+  pieces.reserve(chunks.size() + 2 * W * (bounds.size() - 1));
+  rec_mul.reserve(pieces.capacity());
   for (size_t b = 0; b + 1 < bounds.size(); ++b) {
     BatchInfo bi;
     bi.c_begin = bounds[b];
     bi.c_end = bounds[b + 1];
-    uint64_t class_blocks[kClassCount] = {0, 0, 0, 0, 0, 0};
-    for (uint64_t c = bi.c_begin; c < bi.c_end; ++c) {
-      ChunkDesc& d = chunks[c];
-      d.blk_begin = class_blocks[d.sweep_class];
-      class_blocks[d.sweep_class] += d.len / kBlockBytes;
-    }
-    // the batch's classes: chunk lists and, per class, the class-stream block
-    // where each segment starts (warp ranges start on segment boundaries)
-    struct Cls {
-      uint32_t cls;
-      uint64_t list_off;
-      std::vector<uint64_t> seg_start;
-      std::vector<uint64_t> cost;  // cost[s]: estimated cost of segments [0, s)
-    };
-    std::vector<Cls> cl;
-    for (uint32_t cls = 0; cls < kClassCount; ++cls) {
-      if (class_blocks[cls] == 0) continue;
-      Cls q;
-      q.cls = cls;
-      q.list_off = lists.size();
-      for (uint64_t c = bi.c_begin; c < bi.c_end; ++c)
-        if (chunks[c].sweep_class == cls && chunks[c].len >= static_cast<uint64_t>(kBlockBytes))
-          lists.push_back(static_cast<uint32_t>(c));
-      q.cost.push_back(0);
-      for (size_t i = q.list_off; i < lists.size(); ++i) {
-        const ChunkDesc& d = chunks[lists[i]];
-        const uint64_t nb = d.len / kBlockBytes;
-        for (uint64_t j = 0; j < nb; j += kSegBlocks) {
-          q.seg_start.push_back(d.blk_begin + j);
-          const uint64_t blocks = std::min<uint64_t>(kSegBlocks, nb - j);
-          q.cost.push_back(q.cost.back() + seg_cost(blocks, j == 0));
-        }
-      }
-      q.seg_start.push_back(class_blocks[cls]);
-      cl.push_back(std::move(q));
-    }
     bi.warp_off = warps.size();
     bi.unit_off = units.size();
-    if (cl.empty()) {
-      D.batches.push_back(bi);
-      continue;
+    uint64_t blocks[kClassCount] = {}, segs[kClassCount] = {};
+    for (std::vector<uint32_t>& l : lists) l.clear();
+    for (uint64_t c = bi.c_begin; c < bi.c_end; ++c) {
+      const ChunkDesc& d = chunks[c];
+      const uint64_t nb = d.len / kBlockBytes;
+      if (nb == 0) continue;
+      lists[d.sweep_class].push_back(static_cast<uint32_t>(c));
+      blocks[d.sweep_class] += nb;
+      segs[d.sweep_class] += (nb + kSegBlocks - 1) / kSegBlocks;
     }
-    bi.any = true;
-    // warps per class; slot[q * W + j] = the batch-warp index of class q's j-th warp
-    std::vector<uint64_t> wc(cl.size(), W);
-    std::vector<uint32_t> slot(cl.size() * W);
-    double cost[kClassCount];
-    for (size_t q = 0; q < cl.size(); ++q)
-      cost[q] = static_cast<double>(class_blocks[cl[q].cls]) * class_weight(cl[q].cls, share);
-    share_warps(cost, static_cast<int>(cl.size()), W, wc.data());
+    // the batch's classes, and their warps: slot[q * W + j] = the batch-warp index of class q's j-th
     uint32_t cls_of[kClassCount];
-    for (size_t q = 0; q < cl.size(); ++q) cls_of[q] = cl[q].cls;
-    place_warps(cls_of, wc.data(), static_cast<int>(cl.size()), warps_per_cta, slot.data(), W);
-    warps.resize(bi.warp_off + W);
-    for (size_t q = 0; q < cl.size(); ++q) {
-      const uint32_t cls = cl[q].cls;
-      const size_t lbase = cl[q].list_off;
-      const std::vector<uint64_t>& seg_start = cl[q].seg_start;
-      const uint64_t n_seg = seg_start.size() - 1, Wq = wc[q];
-      const uint64_t n_fix = n_seg - claimed_segs(n_seg, Wq, share);  // segments in the warps' ranges
-      uint64_t k = 0;  // walks the class list monotonically
-      // class blocks [b0, b1) as a run: one piece (and record) per chunk they overlap
-      auto range = [&](uint64_t b0, uint64_t b1) {
+    double cost[kClassCount];
+    uint64_t wc[kClassCount];
+    int n_cls = 0;
+    for (uint32_t cls = 0; cls < kClassCount; ++cls) {
+      if (blocks[cls] == 0) continue;
+      cls_of[n_cls] = cls;
+      cost[n_cls++] = static_cast<double>(blocks[cls]) * class_weight(cls, share);
+    }
+    bi.any = n_cls > 0;
+    if (bi.any) {
+      share_warps(cost, n_cls, W, wc);
+      place_warps(cls_of, wc, n_cls, warps_per_cta, slot.data(), W);
+      warps.resize(bi.warp_off + W);
+    }
+    for (int q = 0; q < n_cls; ++q) {
+      const uint32_t cls = cls_of[q];
+      const uint64_t n_seg = segs[cls], Wq = wc[q];
+      const uint64_t n_fix = n_seg - claimed_segs(n_seg, Wq, share);  // segments in the warps' runs
+      SegWalk at(chunks.data(), lists[cls].data(), lists[cls].size());
+      SegWalk fixed = at;
+      fixed.skip(n_fix);
+      const uint64_t total = fixed.cost();
+      auto run = [&](const SegWalk& to) {
         RunDesc rd;
         rd.first = static_cast<uint32_t>(pieces.size());
+        rd.n = at.emit(to, rd.first, add_piece);
         rd.cls = cls;
         rd.unused = 0;
-        while (b0 < b1) {
-          const uint32_t id = lists[lbase + k];
-          ChunkDesc& d = chunks[id];
-          const uint64_t off = b0 - d.blk_begin, nb = d.len / kBlockBytes;
-          if (off == nb) {
-            ++k;
-            continue;
-          }
-          const uint64_t n = std::min(b1 - b0, nb - off);
-          if (d.n_recs == 0) d.first_rec = static_cast<uint32_t>(pieces.size());
-          d.n_recs += 1;
-          PieceDesc pd;
-          pd.addr = d.addr + off * kBlockBytes;
-          pd.payload_off = d.payload_off + off * kBlockBytes;
-          pd.seg = d.seg_base + static_cast<uint32_t>(off / kSegBlocks);
-          pd.nblk = static_cast<uint32_t>(n);
-          pd.chunk = id;
-          pd.unused = 0;
-          pieces.push_back(pd);
-          rec_mul.push_back(host_xpow8((nb - off - n) * kBlockBytes));
-          b0 += n;
-        }
-        rd.n = static_cast<uint32_t>(pieces.size()) - rd.first;
+        at = to;
         return rd;
       };
-      // the warps' ranges: the first n_fix segments cut by estimated cost
-      std::vector<uint64_t> bnd(Wq + 1);
-      const std::vector<uint64_t>& cost = cl[q].cost;
-      split_ranges([&](uint64_t i) { return cost[i]; }, n_fix, Wq, bnd.data());
-      for (uint64_t w = 0; w < Wq; ++w)
-        warps[bi.warp_off + slot[q * W + w]] = range(seg_start[bnd[w]], seg_start[bnd[w + 1]]);
-      for (uint64_t u = n_fix; u < n_seg;) {
-        const uint64_t n = unit_segs(n_seg - u, Wq);
-        units.push_back(range(seg_start[u], seg_start[u + n]));
-        u += n;
+      for (uint64_t w = 1; w <= Wq; ++w) {
+        SegWalk to = at;
+        to.to_cost(static_cast<uint64_t>(static_cast<unsigned __int128>(total) * w / Wq), n_fix);
+        warps[bi.warp_off + slot[q * W + w - 1]] = run(to);
+      }
+      while (at.segs() < n_seg) {
+        SegWalk to = at;
+        to.skip(unit_segs(n_seg - at.segs(), Wq));
+        units.push_back(run(to));
       }
     }
     bi.n_units = static_cast<uint32_t>(units.size() - bi.unit_off);
     D.batches.push_back(bi);
   }
   D.n_recs = pieces.size();
-  cudaError_t e = upload(&D.d_chunks, chunks);
-  if (e == cudaSuccess) e = upload(&D.d_warps, warps);
-  if (e == cudaSuccess) e = upload(&D.d_pieces, pieces);
-  if (e == cudaSuccess) e = upload(&D.d_rec_mul, rec_mul);
-  if (e == cudaSuccess) e = upload(&D.d_units, units);
-  if (e == cudaSuccess && !units.empty())
-    e = upload(&D.d_queue, std::vector<uint32_t>(kQueueWords * D.batches.size(), 0));
-  const uint64_t slots = std::max<uint64_t>(D.n_recs, min_recs);
-  if (e == cudaSuccess && slots) e = cudaMalloc(&D.d_recs, slots * sizeof(Record));
-  return e;
+  mem.table(&D.d_chunks, chunks);
+  mem.table(&D.d_pieces, pieces);
+  mem.table(&D.d_warps, warps);
+  mem.table(&D.d_rec_mul, rec_mul);
+  mem.table(&D.d_units, units);
+  if (!units.empty()) mem.table(&D.d_queue, std::vector<uint32_t>(kQueueWords * D.batches.size(), 0));
+  mem.scratch(&D.d_recs, std::max<uint64_t>(D.n_recs, min_recs));
+}
+
+// The chunks, layout, tables and device memory of a plan whose sizes are set.
+// On failure (or an exception) the caller frees what there is.
+fr_status fill_plan(fr_plan p, const fr_tensor* tensors, uint64_t n_tensors) {
+  const uint64_t n_chunks = p->n_chunks, chunk_bytes = p->chunk_bytes;
+  // ---- chunks and packed layout
+  p->chunks.resize(n_chunks);
+  uint64_t payload = align_up(n_chunks * kHeaderBytes, kPayloadAlign);
+  uint64_t c = 0;
+  for (uint64_t t = 0; t < n_tensors; ++t) {
+    for (uint64_t off = 0; off < tensors[t].nbytes; off += chunk_bytes) {
+      ChunkDesc& d = p->chunks[c++];
+      std::memset(&d, 0, sizeof d);
+      d.len = std::min<uint64_t>(chunk_bytes, tensors[t].nbytes - off);
+      d.addr = reinterpret_cast<uint64_t>(tensors[t].ptr) + off;
+      d.tensor_off = off;
+      d.payload_off = payload;
+      d.tensor_idx = static_cast<uint32_t>(t);
+      d.dtype = tensors[t].dtype;
+      d.sweep_class = d.dtype * 2 + (d.addr % 16 == 0 ? 1 : 0);
+      d.seg_base = static_cast<uint32_t>(p->n_segs);
+      p->n_segs += (d.len / kBlockBytes + kSegBlocks - 1) / kSegBlocks;
+      payload += align_up(d.len, kPayloadAlign);
+    }
+  }
+  p->packed_bytes = payload;
+  if (p->n_segs >= (1ull << 32)) return invalid("state too large");
+
+  // ---- decompositions
+  PlanMemory mem;
+  if (n_chunks > 0) {
+    // distinct decompositions of the modes: warps per CTA and class weights;
+    // the fingerprint's is geo 0
+    std::vector<int> counts;  // 3 * warps + weights
+    for (int m = 0; m < 4; ++m) {
+      const int w = 3 * sweep_warps(m) + (m == kModeFingerprint ? kShareFingerprint : kSharePack);
+      int g = 0;
+      while (g < static_cast<int>(counts.size()) && counts[g] != w) ++g;
+      if (g == static_cast<int>(counts.size())) counts.push_back(w);
+      p->geo[m] = g;
+    }
+    p->whole.resize(counts.size());
+    p->batched.resize(counts.size());
+    for (size_t g = 0; g < counts.size(); ++g)
+      build_decomp(p->chunks, {0, n_chunks}, p->n_sm, counts[g] / 3, counts[g] % 3, g == 0 ? n_chunks : 0, p->whole[g], mem);
+    if (p->n_batches > 1) {
+      // batch starts at about equal state bytes, every batch non-empty
+      std::vector<uint64_t> bounds(1, 0);
+      uint64_t acc = 0, cc = 0;
+      for (uint32_t b = 1; b < p->n_batches; ++b) {
+        const uint64_t target = p->state_bytes / p->n_batches * b;
+        while (cc < n_chunks && (acc < target || cc <= bounds.back())) acc += p->chunks[cc++].len;
+        const uint64_t room = n_chunks - (p->n_batches - b);  // leave one chunk per later batch
+        bounds.push_back(std::min(cc, room));
+      }
+      bounds.push_back(n_chunks);
+      for (size_t i = 1; i < bounds.size(); ++i)
+        if (bounds[i] <= bounds[i - 1]) bounds[i] = bounds[i - 1] + 1;
+      for (size_t g = 0; g < counts.size(); ++g) {
+        bool used = false;  // no call fingerprints a batch
+        for (int m = 0; m < 4; ++m) used |= m != kModeFingerprint && p->geo[m] == static_cast<int>(g);
+        if (used)
+          build_decomp(p->chunks, bounds, std::max(1, p->n_sm / 2), counts[g] / 3, counts[g] % 3, 0, p->batched[g], mem);
+      }
+    }
+  }
+  std::vector<uint32_t> crc_xor(n_chunks);
+  for (uint64_t c = 0; c < n_chunks; ++c)
+    crc_xor[c] = c > 0 && p->chunks[c].len == p->chunks[c - 1].len ? crc_xor[c - 1] : host_crc_xor_term(p->chunks[c].len);
+  mem.table(&p->d_crc_xor, crc_xor);
+  mem.table(&p->d_status, std::vector<uint32_t>(1, 0));
+  mem.scratch(&p->d_segs, p->n_segs);
+  mem.scratch(&p->d_flags, n_chunks);
+  mem.scratch(&p->d_ids, n_chunks);
+  mem.scratch(&p->d_count, 1);
+  cudaError_t e = mem.commit(&p->d_memory);
+  for (uint32_t i = 0; e == cudaSuccess && i < p->n_batches + 1; ++i) {
+    cudaEvent_t ev;
+    e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) p->events.push_back(ev);
+  }
+  return e == cudaSuccess ? FR_OK : cuda_fail(e, "plan device tables");
 }
 
 // Sweep + finalize of batches [b0, b1) of decomposition D.
@@ -545,86 +598,15 @@ fr_status fr_plan_create_batched(const fr_tensor* tensors, uint64_t n_tensors, u
   p->state_bytes = state;
   p->n_batches = static_cast<uint32_t>(std::max<uint64_t>(1, std::min<uint64_t>(n_batches, n_chunks)));
 
-  // ---- chunks and packed layout
-  p->chunks.resize(n_chunks);
-  uint64_t payload = align_up(n_chunks * kHeaderBytes, kPayloadAlign);
-  uint64_t c = 0;
-  for (uint64_t t = 0; t < n_tensors; ++t) {
-    for (uint64_t off = 0; off < tensors[t].nbytes; off += chunk_bytes) {
-      ChunkDesc& d = p->chunks[c++];
-      std::memset(&d, 0, sizeof d);
-      d.len = std::min<uint64_t>(chunk_bytes, tensors[t].nbytes - off);
-      d.addr = reinterpret_cast<uint64_t>(tensors[t].ptr) + off;
-      d.tensor_off = off;
-      d.payload_off = payload;
-      d.tensor_idx = static_cast<uint32_t>(t);
-      d.dtype = tensors[t].dtype;
-      d.sweep_class = d.dtype * 2 + (d.addr % 16 == 0 ? 1 : 0);
-      d.seg_base = static_cast<uint32_t>(p->n_segs);
-      p->n_segs += (d.len / kBlockBytes + kSegBlocks - 1) / kSegBlocks;
-      payload += align_up(d.len, kPayloadAlign);
-    }
+  try {
+    st = fill_plan(p, tensors, n_tensors);
+  } catch (const std::bad_alloc&) {
+    st = invalid("out of host memory");
   }
-  p->packed_bytes = payload;
-  if (p->n_segs >= (1ull << 32)) {
-    delete p;
-    return invalid("state too large");
-  }
-
-  // ---- decompositions
-  e = cudaSuccess;
-  if (n_chunks > 0) {
-    // distinct decompositions of the modes: warps per CTA and class weights;
-    // the fingerprint's is geo 0
-    std::vector<int> counts;  // 3 * warps + weights
-    for (int m = 0; m < 4; ++m) {
-      const int w = 3 * sweep_warps(m) + (m == kModeFingerprint ? kShareFingerprint : kSharePack);
-      int g = 0;
-      while (g < static_cast<int>(counts.size()) && counts[g] != w) ++g;
-      if (g == static_cast<int>(counts.size())) counts.push_back(w);
-      p->geo[m] = g;
-    }
-    p->whole.resize(counts.size());
-    p->batched.resize(counts.size());
-    for (size_t g = 0; e == cudaSuccess && g < counts.size(); ++g)
-      e = build_decomp(p->chunks, {0, n_chunks}, n_sm, counts[g] / 3, counts[g] % 3, g == 0 ? n_chunks : 0, p->whole[g]);
-    if (e == cudaSuccess && p->n_batches > 1) {
-      // batch starts at about equal state bytes, every batch non-empty
-      std::vector<uint64_t> bounds(1, 0);
-      uint64_t acc = 0, cc = 0;
-      for (uint32_t b = 1; b < p->n_batches; ++b) {
-        const uint64_t target = state / p->n_batches * b;
-        while (cc < n_chunks && (acc < target || cc <= bounds.back())) acc += p->chunks[cc++].len;
-        const uint64_t room = n_chunks - (p->n_batches - b);  // leave one chunk per later batch
-        bounds.push_back(std::min(cc, room));
-      }
-      bounds.push_back(n_chunks);
-      for (size_t i = 1; i < bounds.size(); ++i)
-        if (bounds[i] <= bounds[i - 1]) bounds[i] = bounds[i - 1] + 1;
-      for (size_t g = 0; e == cudaSuccess && g < counts.size(); ++g)
-        e = build_decomp(p->chunks, bounds, std::max(1, n_sm / 2), counts[g] / 3, counts[g] % 3, 0, p->batched[g]);
-    }
-  }
-  if (e == cudaSuccess && p->n_segs) e = cudaMalloc(&p->d_segs, p->n_segs * sizeof(double));
-  if (e == cudaSuccess && n_chunks) {
-    std::vector<uint32_t> crc_xor(n_chunks);
-    for (uint64_t c = 0; c < n_chunks; ++c) crc_xor[c] = host_crc_xor_term(p->chunks[c].len);
-    e = upload(&p->d_crc_xor, crc_xor);
-  }
-  if (e == cudaSuccess && n_chunks) e = cudaMalloc(&p->d_flags, n_chunks);
-  if (e == cudaSuccess && n_chunks) e = cudaMalloc(&p->d_ids, n_chunks * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&p->d_count, sizeof(uint64_t));
-  if (e == cudaSuccess) e = cudaMalloc(&p->d_status, sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, sizeof(uint32_t));
-  for (uint32_t i = 0; e == cudaSuccess && i < p->n_batches + 1; ++i) {
-    cudaEvent_t ev;
-    e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-    if (e == cudaSuccess) p->events.push_back(ev);
-  }
-  if (e != cudaSuccess) {
+  if (st != FR_OK) {
     free_device(p);
     delete p;
-    return cuda_fail(e, "plan device tables");
+    return st;
   }
   *out = p;
   return FR_OK;

@@ -62,7 +62,7 @@ struct ChunkDesc {       // 64 bytes
   uint64_t len;          // chunk bytes
   uint64_t tensor_off;   // offset of the chunk inside its tensor
   uint64_t payload_off;  // offset of the payload in the packed buffer
-  uint64_t blk_begin;    // first body block in its class's block stream (planning only)
+  uint64_t unused;
   uint32_t tensor_idx;
   uint32_t dtype;
   uint32_t first_rec;    // records of this chunk: [first_rec, first_rec + n_recs)

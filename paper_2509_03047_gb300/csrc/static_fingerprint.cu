@@ -30,6 +30,7 @@
 #include "gf2.cuh"
 #include "kernels.h"
 #include "layout.h"
+#include "seg_walk.h"
 #include "warp_share.h"
 
 using namespace frk;
@@ -60,12 +61,9 @@ static __device__ __align__(256) uint8_t g_static_scratch[kScratchBytes];
 // Host copies of the tables, staged here and copied into the scratch.
 struct HostTables {
   ChunkDesc chunks[kMaxChunks];
-  uint32_t lists[kMaxChunks];  // per class: its chunks with a body, in order
+  uint32_t list[kMaxChunks];  // of one class: its chunks with a body, in order
   RunDesc warps[kMaxWarps];
   PieceDesc pieces[kMaxRecs];
-  uint64_t seg_start[kMaxSegs + 1];  // per class: block where each segment starts
-  uint64_t seg_cost[kMaxSegs + 1];   // per class: estimated cost of its segments before each
-  uint64_t bnd[kMaxWarps + 1];       // per class: the segment where each warp's range starts
   uint32_t slot[kClasses * kMaxWarps];  // per class: launch-warp index of its j-th warp
 };
 HostTables g_host;
@@ -150,7 +148,7 @@ extern "C" fr_status fr_fingerprint_static(const fr_tensor* tensors, uint64_t n_
   // ---- plan into the static host tables (same rules as fr_plan_create)
   HostTables& h = g_host;
   uint64_t payload = align_up(n_chunks * kHeaderBytes, kPayloadAlign);
-  uint64_t class_blocks[kClasses] = {0, 0, 0, 0, 0, 0};
+  uint64_t class_blocks[kClasses] = {}, class_segs[kClasses] = {};
   uint64_t c = 0, seg = 0;
   for (uint64_t t = 0; t < n_tensors; ++t) {
     for (uint64_t off = 0; off < tensors[t].nbytes; off += chunk_bytes) {
@@ -160,14 +158,14 @@ extern "C" fr_status fr_fingerprint_static(const fr_tensor* tensors, uint64_t n_
       d.addr = reinterpret_cast<uint64_t>(tensors[t].ptr) + off;
       d.tensor_off = off;
       d.payload_off = payload;
-            d.tensor_idx = static_cast<uint32_t>(t);
+      d.tensor_idx = static_cast<uint32_t>(t);
       d.dtype = tensors[t].dtype;
       d.sweep_class = d.dtype * 2 + (d.addr % 16 == 0 ? 1 : 0);
       d.seg_base = static_cast<uint32_t>(seg);
       seg += (d.len / kBlockBytes + kSegBlocks - 1) / kSegBlocks;
       payload += align_up(d.len, kPayloadAlign);
-      d.blk_begin = class_blocks[d.sweep_class];
       class_blocks[d.sweep_class] += d.len / kBlockBytes;
+      class_segs[d.sweep_class] += (d.len / kBlockBytes + kSegBlocks - 1) / kSegBlocks;
     }
   }
   // one launch for every class: the W warps shared by weighted blocks, each
@@ -186,56 +184,26 @@ extern "C" fr_status fr_fingerprint_static(const fr_tensor* tensors, uint64_t n_
     share_warps(cost, n_cls, W, wc);
     place_warps(cls_of, wc, n_cls, sweep_warps(kModeFingerprint), h.slot, kMaxWarps);
   }
-  uint64_t n_lists = 0, n_recs = 0;
+  uint64_t n_recs = 0;
   for (int q = 0; q < n_cls; ++q) {
     const uint32_t cls = cls_of[q];
-    const uint64_t blk = class_blocks[cls], Wq = wc[q];
-    const uint64_t list_off = n_lists;
+    uint64_t n_list = 0;
     for (uint64_t i = 0; i < n_chunks; ++i)
       if (h.chunks[i].sweep_class == cls && h.chunks[i].len >= static_cast<uint64_t>(kBlockBytes))
-        h.lists[n_lists++] = static_cast<uint32_t>(i);
-    const uint32_t* list = h.lists + list_off;
-    // warp ranges start on 16 KiB segment boundaries (see layout.h)
-    uint64_t n_class_segs = 0;
-    h.seg_cost[0] = 0;
-    for (uint64_t i = list_off; i < n_lists; ++i) {
-      const ChunkDesc& d = h.chunks[h.lists[i]];
-      const uint64_t nb = d.len / kBlockBytes;
-      for (uint64_t j = 0; j < nb; j += kSegBlocks) {
-        h.seg_start[n_class_segs] = d.blk_begin + j;
-        h.seg_cost[n_class_segs + 1] = h.seg_cost[n_class_segs] + seg_cost(std::min<uint64_t>(kSegBlocks, nb - j), j == 0);
-        ++n_class_segs;
-      }
-    }
-    h.seg_start[n_class_segs] = blk;
-    split_ranges([&](uint64_t s) { return h.seg_cost[s]; }, n_class_segs, Wq, h.bnd);
-    uint64_t k = 0;
-    for (uint64_t w = 0; w < Wq; ++w) {
-      const uint64_t b0 = h.seg_start[h.bnd[w]], b1 = h.seg_start[h.bnd[w + 1]];
-      RunDesc& rd = h.warps[h.slot[q * kMaxWarps + w]];
+        h.list[n_list++] = static_cast<uint32_t>(i);
+    SegWalk at(h.chunks, h.list, n_list), end = at;
+    end.skip(class_segs[cls]);
+    const uint64_t total = end.cost();
+    for (uint64_t w = 1; w <= wc[q]; ++w) {
+      SegWalk to = at;
+      to.to_cost(total * w / wc[q], class_segs[cls]);
+      RunDesc& rd = h.warps[h.slot[q * kMaxWarps + w - 1]];
       rd.first = static_cast<uint32_t>(n_recs);
+      // n_recs <= W + chunks <= kMaxRecs
+      rd.n = at.emit(to, rd.first, [&](const PieceDesc& pd, uint64_t) { h.pieces[n_recs++] = pd; });
       rd.cls = cls;
       rd.unused = 0;
-      for (uint64_t b = b0; b < b1;) {
-        ChunkDesc& d = h.chunks[list[k]];
-        const uint64_t off = b - d.blk_begin, nb = d.len / kBlockBytes;
-        if (off == nb) {
-          ++k;
-          continue;
-        }
-        const uint64_t n = std::min(b1 - b, nb - off);
-        if (d.n_recs == 0) d.first_rec = static_cast<uint32_t>(n_recs);
-        d.n_recs += 1;
-        PieceDesc& pd = h.pieces[n_recs++];  // n_recs <= W + chunks <= kMaxRecs
-        pd.addr = d.addr + off * kBlockBytes;
-        pd.payload_off = d.payload_off + off * kBlockBytes;
-        pd.seg = d.seg_base + static_cast<uint32_t>(off / kSegBlocks);
-        pd.nblk = static_cast<uint32_t>(n);
-        pd.chunk = list[k];
-        pd.unused = 0;
-        b += n;
-      }
-      rd.n = static_cast<uint32_t>(n_recs) - rd.first;
+      at = to;
     }
   }
   const uint64_t n_warps = n_cls > 0 ? W : 0;

@@ -14,8 +14,8 @@
 //    advanced by s <- (s ^ w) * x^4096 with four byte lookups in tables kept in
 //    shared memory.  Every lane has a private copy of each table entry in its
 //    own bank, so the 32 lookups of a warp never conflict.  At the end of a
-//    piece the streams are folded with GF(2) multiplications by constants and
-//    warp shuffles into the raw CRC of the piece;
+//    piece each lane's streams are multiplied to their place and XORed into the
+//    raw CRC of the piece;
 //  * non-finite count and sum of squares, fused on the same registers: each
 //    square is added to a packed f32x2 running sum by one FMA, and the
 //    addition's error -- including the square's own rounding for fp32 -- is
@@ -66,7 +66,7 @@ constexpr int kTableBytes = 4 * 256 * 32 * 4;  // 4 tables x 256 entries x 32 la
 #endif
 // The fingerprint of shifted chunks takes the shorter stage: its loop holds
 // the realignment too, and with 8-block stages the loops of two element types
-// outgrow the instruction cache (2.5 GB of views: 686 us, 597 with 4).
+// outgrow the instruction cache (2.5 GB of views: 567 us, 560 with 4).
 #ifndef FR_STAGE_FP_SHIFT
 #define FR_STAGE_FP_SHIFT 4
 #endif
@@ -148,32 +148,64 @@ __device__ __forceinline__ uint32_t braid_step(uint32_t x, uint32_t lb) {
   return (t0 ^ t1) ^ (t2 ^ t3);
 }
 
-// The piece-end fold multiplies by seven constants: x^32 (Horner inside the
-// lane), x^128 ... x^2048 (the shuffle tree) and the unbraid factor.  Each
-// multiply is four byte lookups in that constant's tables (read-only, cached
-// in L1) instead of a 32-step bit loop: a warp pays the fold once per piece,
-// which matters for states of many small tensors.
-struct FoldTables {
-  ByteTables4 m[7];
-};
-__host__ __device__ constexpr FoldTables make_fold_tables() {
-  FoldTables f{};
-  f.m[0] = make_mul_tables(gf_xpow(32));
-  f.m[1] = make_mul_tables(gf_xpow(128));
-  f.m[2] = make_mul_tables(gf_xpow(256));
-  f.m[3] = make_mul_tables(gf_xpow(512));
-  f.m[4] = make_mul_tables(gf_xpow(1024));
-  f.m[5] = make_mul_tables(gf_xpow(2048));
-  f.m[6] = make_mul_tables(kUnbraid);
-  return f;
-}
-__device__ const FoldTables g_fold = make_fold_tables();
+// The piece-end fold.  A lane joins its four streams by Horner with x^32, then
+// multiplies by x^(128 (31 - l)), its place among the lanes, and by the
+// unbraid factor at once, and the lanes are XORed.  x^32 comes from byte
+// tables (read-only, in L1).  The product (n << 4k) * M_l, for nibble position
+// k, nibble value n and lane l's multiplier M_l, sits at word
+// (16k + n) * 32 + l of a 16 KiB table behind the braid tables in shared
+// memory: the 32 lanes' lookups of a nibble position fall in 32 banks.  A warp
+// pays the fold once per piece; as a tree of five shuffles and multiplications
+// by byte tables, 24 lookups of up to 8 lines each, it was as much load/store
+// work as 10 blocks (40,000 chunks of 1.5 KB on average: step 253 -> 243 us).
+__device__ const ByteTables4 g_x32 = make_mul_tables(gf_xpow(32));
 
-// a * (constant i) mod P.
-__device__ __forceinline__ uint32_t mul_fold(int i, uint32_t a) {
-  const ByteTables4& T = g_fold.m[i];
-  return (__ldg(&T.t[0][a & 255u]) ^ __ldg(&T.t[1][(a >> 8) & 255u])) ^
-         (__ldg(&T.t[2][(a >> 16) & 255u]) ^ __ldg(&T.t[3][a >> 24]));
+constexpr int kLaneFoldWords = 8 * 16 * 32;
+struct alignas(16) LaneFoldTable {
+  uint32_t t[kLaneFoldWords];
+};
+__host__ __device__ constexpr LaneFoldTable make_lane_fold_table() {
+  LaneFoldTable out{};
+  for (int l = 0; l < 32; ++l) {
+    const uint32_t m = gf_mulmod(gf_xpow(128ull * static_cast<uint64_t>(31 - l)), kUnbraid);
+    for (int k = 0; k < 8; ++k) {
+      uint32_t bit[4] = {};
+      for (int j = 0; j < 4; ++j) bit[j] = gf_mulmod(1u << (4 * k + j), m);
+      for (int n = 0; n < 16; ++n) {
+        uint32_t v = 0;
+        for (int j = 0; j < 4; ++j)
+          if (n & (1 << j)) v ^= bit[j];
+        out.t[(16 * k + n) * 32 + l] = v;
+      }
+    }
+  }
+  return out;
+}
+__device__ const LaneFoldTable g_lane_fold = make_lane_fold_table();
+constexpr int kSweepSmem = kTableBytes + kLaneFoldWords * 4;
+
+// Starts this thread's share of the lane table on its way to shared memory;
+// fill_tables waits for it.
+template <int kThreads>
+__device__ __forceinline__ void start_lane_fold() {
+  const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(g_smem + kTableBytes));
+  for (int q = static_cast<int>(threadIdx.x); q < kLaneFoldWords / 4; q += kThreads)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(base + 16u * q), "l"(g_lane_fold.t + 4 * q) : "memory");
+}
+__device__ __forceinline__ void finish_lane_fold() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// a * x^32 mod P.
+__device__ __forceinline__ uint32_t mul_x32(uint32_t a) {
+  return (__ldg(&g_x32.t[0][a & 255u]) ^ __ldg(&g_x32.t[1][(a >> 8) & 255u])) ^
+         (__ldg(&g_x32.t[2][(a >> 16) & 255u]) ^ __ldg(&g_x32.t[3][a >> 24]));
+}
+// a * M_l mod P for the calling lane l (lb = 4l).
+__device__ __forceinline__ uint32_t mul_lane(uint32_t a, uint32_t lb) {
+  const uint8_t* T = g_smem + kTableBytes + lb;
+  uint32_t r[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) r[k] = *reinterpret_cast<const uint32_t*>(T + (16 * k + ((a >> (4 * k)) & 15u)) * 128);
+  return (r[0] ^ r[1] ^ r[2]) ^ (r[3] ^ r[4] ^ r[5]) ^ (r[6] ^ r[7]);
 }
 
 // ------------------------------------------------------------------ memory
@@ -187,6 +219,13 @@ __device__ __forceinline__ uint4 ld_unit(const uint8_t* p) {
   return v;
 }
 
+// The same, kept in L1 for the neighbour lane.
+__device__ __forceinline__ uint4 ld_unit_l1(const uint8_t* p) {
+  uint4 v;
+  asm("ld.global.nc.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
 __device__ __forceinline__ void st_unit(uint8_t* p, const uint4& v) {
   asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z),
                "r"(v.w)
@@ -194,20 +233,25 @@ __device__ __forceinline__ void st_unit(uint8_t* p, const uint4& v) {
 }
 
 // Chunks that do not start on a 16-byte boundary move in 16-byte granules all
-// the same.  A lane's unit lies across two granules.  Reading, lane l loads
-// the one its unit ends in and gets the one it starts in from lane l - 1 by
-// shuffle (lane 0: from lane 31's of the block before); take16 cuts the unit
-// out.  Writing, lane l stores the granule its unit starts in, whose first
-// bytes are the end of lane l - 1's unit.  So every lane holds the same 16
-// bytes of the chunk as for an aligned chunk, and neither the CRC streams nor
-// the order of the sums change with the alignment.  A granule is only read if
-// it holds a byte of the piece, so no read reaches a page that the tensor does
-// not; its other bytes are dropped, and never written.
+// the same.  Reading, a lane's unit lies across two granules of the tensor:
+// lane l loads the one it ends in, as part of the block's pipeline, and the one
+// it starts in -- lane l - 1's, or lane 31's of the block before -- again from
+// L1 when it needs it; take16 cuts the unit out.  Writing, lane l stores the
+// granule its unit starts in, whose first bytes are the end of the unit before
+// it, taken from the packed buffer in the same way.  So every lane holds the
+// same 16 bytes of the chunk as for an aligned chunk, and neither the CRC
+// streams nor the order of the sums change with the alignment.  A granule of
+// the tensor is only read if it holds a byte of the piece, so no read reaches
+// a page that the tensor does not; its other bytes are dropped, and never
+// written.
 //
 // Before, such chunks moved by 4-byte or single-byte accesses 16 bytes apart
 // from lane to lane: 4 or 16 times the load and store instructions, each
-// touching every line of the block.  GB300, 2.5 GB of views at any element
-// offset, us: fingerprint 1095 -> 597, pack 1025 -> 931, unpack 1495 -> 791.
+// touching every line of the block.  With the neighbour's granule passed by
+// shuffle instead of L1 (four shuffles, a carry and a select each) the loops
+// were 12 instructions a block longer.  GB300, 2.5 GB of views at any element
+// offset, us, by narrow accesses / shuffles / L1: fingerprint 1095 / 597 / 529,
+// pack 1025 / 931 / 783, pack and unpack with both tables 2063 / 1917 / 1610.
 
 // 16 bytes from byte t on (0 <= t < 16, the same in every lane) of a then b.
 __device__ __forceinline__ uint4 take16(const uint4& a, const uint4& b, uint32_t t) {
@@ -230,15 +274,6 @@ __device__ __forceinline__ uint4 take16(const uint4& a, const uint4& b, uint32_t
   const uint32_t sh = 8u * (t & 3u);
   return make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh), __funnelshift_r(w2, w3, sh),
                     __funnelshift_r(w3, w4, sh));
-}
-
-// Lane `from`'s v.
-__device__ __forceinline__ uint4 shfl4(const uint4& v, uint32_t from) {
-  return make_uint4(__shfl_sync(0xFFFFFFFFu, v.x, from), __shfl_sync(0xFFFFFFFFu, v.y, from),
-                    __shfl_sync(0xFFFFFFFFu, v.z, from), __shfl_sync(0xFFFFFFFFu, v.w, from));
-}
-__device__ __forceinline__ uint4 select4(bool c, const uint4& a, const uint4& b) {
-  return make_uint4(c ? a.x : b.x, c ? a.y : b.y, c ? a.z : b.z, c ? a.w : b.w);
 }
 
 // The unit at p by itself; SHIFT: p need not be a multiple of 16.
@@ -538,19 +573,18 @@ struct Lane {
   FpAcc f;        // fp32 sums of the current span
   uint32_t nonfinite;
   // shifted pieces only
-  uint32_t t;     // take16's t
-  uint4 carry;    // lane 0: lane 31's granule (source) or unit (destination) of the previous block
-  bool first;     // destination, lane 0: no block stored yet
+  uint32_t t;  // take16's t
+  bool first;  // destination, lane 0: no block stored yet
 };
 
+// One unit `v`, which goes to wp; `up`: where it was loaded.
 template <int MODE, int DT, bool SHIFT>
-__device__ __forceinline__ void do_unit(Lane<MODE, DT>& L, const uint4& v, uint8_t* wp, uint32_t lb) {
+__device__ __forceinline__ void do_unit(Lane<MODE, DT>& L, const uint4& v, const uint8_t* up, uint8_t* wp, uint32_t lb) {
   constexpr bool kFp = mode_sums(MODE) && (DT != kDtBytes);
   if (MODE != kModeFingerprint) {
     if (SHIFT && mode_unpacks(MODE)) {
-      const uint4 y = shfl4(v, (lb / 4 + 31) & 31u);
-      const uint4 g = take16(select4(lb == 0, L.carry, y), v, L.t);
-      L.carry = y;
+      // (16 bytes before a payload are still in the packed buffer)
+      const uint4 g = take16(ld_unit_l1(up - 16), v, L.t);
       if (!L.first)
         st_unit(wp, g);
       else
@@ -567,28 +601,49 @@ __device__ __forceinline__ void do_unit(Lane<MODE, DT>& L, const uint4& v, uint8
   if (kFp) fp_unit<DT>(v, L.f);
 }
 
-// End of a span (one segment) of `n` blocks, the lane's first unit at sp: the fast sums are kept if finite and
-// either large enough that fp32 underflow is negligible (below 2^-77 relative)
-// or made of zeros only; otherwise the segment is summed exactly from a
-// reload.  The lanes' sums are then added in a fixed tree and lane 0 stores
-// the segment's sum (a float pair, see seg_value) at its index.
-template <int MODE, int DT, bool SHIFT>
-__device__ __forceinline__ void span_end(Lane<MODE, DT>& L, const uint8_t* sp, uint32_t n, double* seg,
-                                         uint32_t lane) {
-  const u64 ab = add2(L.f.A, L.f.B);
-  const float tot = lo_f(ab) + hi_f(ab);
+// The lanes' float pairs added in a fixed tree by TwoSum; lane 0 stores the
+// segment's sum in pair form (seg_value).
+__device__ __forceinline__ void store_pair_sum(float hi, float lo, double* seg, uint32_t lane) {
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) {
+    const float oh = __shfl_down_sync(0xFFFFFFFFu, hi, m);
+    const float ol = __shfl_down_sync(0xFFFFFFFFu, lo, m);
+    const float t = hi + oh;
+    const float z = t - hi;
+    const float err = (hi - (t - z)) + (oh - z);
+    lo = (lo + ol) + err;
+    hi = t;
+  }
+  if (lane == 0) *reinterpret_cast<float2*>(seg) = make_float2(lo, hi);
+}
+
+// End of a segment some lane of which has a running sum `tot` outside
+// [2^-60, 2^120): the lane's fast sums stand if finite and not small (fp32
+// underflow is then below 2^-77 relative), or if its elements are all zero;
+// else the lane's share is summed exactly from a reload.  Lanes that all took
+// the fast path with sums far from fp32 overflow are added in pair form, else
+// in fp64.  Returns the lane's non-finite elements.
+template <int DT, bool SHIFT>
+__device__ __noinline__ uint32_t span_end_slow(FpAcc f, float tot, const uint8_t* sp, uint32_t n, double* seg,
+                                               uint32_t lane) {
   bool ok = tot < __int_as_float(0x7F800000);
   if (ok && !(tot >= 0x1p-60f)) ok = span_is_zero<DT, SHIFT>(sp, n);
   float hi = 0.0f, lo = 0.0f;
   double d = 0.0;
-  if (ok) fold_to_pair(L.f, hi, lo);
+  uint32_t nonfinite = 0;
+  if (ok) fold_to_pair(f, hi, lo);
+  if (__all_sync(0xFFFFFFFFu, ok && tot < 0x1p120f)) {
+    store_pair_sum(hi, lo, seg, lane);
+    return 0;
+  }
+  if (ok) d = static_cast<double>(hi) + static_cast<double>(lo);
   uint32_t bad = __ballot_sync(0xFFFFFFFFu, !ok);
   if (__popc(bad) > kSlowWarpLanes) {
     bad = 0;
     if (!ok) {
       const Exact x = slow_span<DT, SHIFT>(sp, n);
       d = x.d;
-      L.nonfinite += x.nonfinite;
+      nonfinite = x.nonfinite;
     }
   }
   for (; bad != 0; bad &= bad - 1) {
@@ -596,45 +651,50 @@ __device__ __forceinline__ void span_end(Lane<MODE, DT>& L, const uint8_t* sp, u
     const Exact x = slow_span_by_warp<DT, SHIFT>(sp, n, l, lane);
     if (lane == l) {
       d = x.d;
-      L.nonfinite += x.nonfinite;
+      nonfinite = x.nonfinite;
     }
   }
-  L.f.A = L.f.CA = L.f.B = L.f.CB = 0ull;
-  // The lanes' sums are added in a fixed tree: as float pairs by TwoSum when
-  // every lane took the fast path with a sum far from fp32 overflow (no fp64
-  // work), else in fp64 (rare).  Lane 0 stores the form seg_value() reads.
-  if (__all_sync(0xFFFFFFFFu, ok && tot < 0x1p120f)) {
 #pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) {
-      const float oh = __shfl_down_sync(0xFFFFFFFFu, hi, m);
-      const float ol = __shfl_down_sync(0xFFFFFFFFu, lo, m);
-      const float t = hi + oh;
-      const float z = t - hi;
-      const float err = (hi - (t - z)) + (oh - z);
-      lo = (lo + ol) + err;
-      hi = t;
-    }
-    if (lane == 0) *reinterpret_cast<float2*>(seg) = make_float2(lo, hi);
-  } else {
-    if (ok) d = static_cast<double>(hi) + static_cast<double>(lo);
-#pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, m);
-    if (lane == 0) *seg = -d;
-  }
+  for (int m = 16; m >= 1; m >>= 1) d += __shfl_down_sync(0xFFFFFFFFu, d, m);
+  if (lane == 0) *seg = -d;
+  return nonfinite;
 }
 
-// One piece: `nblk` 512-byte blocks from `src` (to `dst` for pack/unpack).
-// SHIFT: the tensor side (source, or destination for unpack) does not start
-// on a 16-byte boundary; the packed side always does.
+// End of a span (one segment) of `n` blocks, the lane's first unit at sp.  The
+// common case in line, all else behind one vote and one call: the loops of two
+// element types only just fit an SM's instruction cache (fingerprint of 4.2 GB
+// in 50,000 tensors 694 -> 679 us, of the Llama-8B shard 2132 -> 2078).
+template <int MODE, int DT, bool SHIFT>
+__device__ __forceinline__ void span_end(Lane<MODE, DT>& L, const uint8_t* sp, uint32_t n, double* seg,
+                                         uint32_t lane) {
+  const u64 ab = add2(L.f.A, L.f.B);
+  const float tot = lo_f(ab) + hi_f(ab);
+  if (__all_sync(0xFFFFFFFFu, tot >= 0x1p-60f && tot < 0x1p120f)) {
+    float hi, lo;
+    fold_to_pair(L.f, hi, lo);
+    store_pair_sum(hi, lo, seg, lane);
+  } else {
+    L.nonfinite += span_end_slow<DT, SHIFT>(L.f, tot, sp, n, seg, lane);
+  }
+  L.f.A = L.f.CA = L.f.B = L.f.CB = 0ull;
+}
+
+// A run of `n` consecutive pieces of one class, a warp's own or a unit it
+// claimed: piece i (from r on) is get(i, whether more
+// follow), its record recs[i].  SHIFT: the
+// tensor side (source, or destination for unpack) of the class's chunks does
+// not start on a 16-byte boundary; the packed side always does.
 //
 // Pipeline: for the fingerprint, lane 0 prefetches whole spans into L2 one span
-// ahead with the bulk-copy unit; each lane keeps kStage 16-byte units of the next stage in
-// flight in registers, which therefore mostly wait for L2.  Each span is one
-// sum segment: its fp32 sums start at zero, are checked at its end, and are
-// replaced by an exact sum from a reload when they fail.
-template <int MODE, int DT, bool SHIFT>
-__device__ __forceinline__ void sweep_piece(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst,
-                                            uint32_t nblk, uint32_t lane, Record* rec, double* seg) {
+// ahead with the bulk-copy unit; each lane keeps kStage 16-byte units of the
+// next stage in flight in registers, which therefore mostly wait for L2.  Each
+// span is one sum segment: its fp32 sums start at zero, are checked at its end,
+// and are replaced by an exact sum from a reload when they fail.  (Loading a
+// piece's first stage before the piece before it is folded gained pack 0.3%
+// and cost the fingerprint of the Llama-8B shard 3%.)
+template <int MODE, int DT, bool SHIFT, class Get>
+__device__ __forceinline__ void sweep_run(uint8_t* packed, double* segs, Record* recs, const Get& get, uint32_t r,
+                                          uint32_t n, uint32_t lane) {
   constexpr bool kFp = mode_sums(MODE) && (DT != kDtBytes);
   constexpr uint32_t kStage = Geo<MODE, SHIFT>::kStage;
   constexpr bool kPrefetch = Geo<MODE, SHIFT>::kPrefetch;
@@ -644,158 +704,139 @@ __device__ __forceinline__ void sweep_piece(const uint8_t* __restrict__ src, uin
   const uint32_t lb = lane << 2;
 
   Lane<MODE, DT> L;
-  L.s[0] = L.s[1] = L.s[2] = L.s[3] = 0;
-  L.f = FpAcc{0ull, 0ull, 0ull, 0ull};
-  L.nonfinite = 0;
-  const uint8_t* lp = src;
-  uint8_t* wp = dst;
-  if (kShiftSrc) {
-    L.t = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(src)) & 15u;
-    lp += 16u - L.t;
-    L.carry = lane == 0 ? ld_unit(lp - 16) : make_uint4(0u, 0u, 0u, 0u);
-  }
-  if (kShiftDst) {
-    const uint32_t before = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(dst)) & 15u;
-    L.t = 16u - before;
-    wp -= before;
-    L.carry = make_uint4(0u, 0u, 0u, 0u);
-    L.first = lane == 0;
-  }
-
-  // The first span goes to L2 now; each later one about a span before use.
-  if (kPrefetch) prefetch_l2_lane0(lp, (nblk < kSpan ? nblk : kSpan) * kBlockBytes, lane);
-
-  // (Every unit is given a value here: a register that is only set under a
-  // condition is live, to the compiler, around every loop that encloses this
-  // one, through the code of every class -- 1,000 bytes of spills.)
+  const uint8_t* lp;  // the next stage's loads
+  uint8_t* wp;
+  uint32_t left;  // blocks not swept yet
+  double* seg;
   uint4 cur[kStage];
-  lp += lane * 16;
-  wp += lane * 16;
+  auto load = [&](const uint8_t* q) { return SHIFT ? ld_unit_l1(q) : ld_unit(q); };
+  // Starts piece r.  (Every unit is given a value: a register that is only set
+  // under a condition is live, to the compiler, around every loop that
+  // encloses this one, through the code of every class -- 1,000 bytes of
+  // spills.)
+  auto begin = [&]() {
+    const PieceDesc d = get(r, n > 1);
+    uint8_t* tensor = reinterpret_cast<uint8_t*>(d.addr);
+    uint8_t* pk = packed + d.payload_off;
+    lp = mode_unpacks(MODE) ? pk : tensor;
+    wp = mode_unpacks(MODE) ? tensor : pk;
+    left = d.nblk;
+    seg = segs + d.seg;
+    if (kShiftSrc) {
+      L.t = static_cast<uint32_t>(d.addr) & 15u;
+      lp += 16u - L.t;
+    }
+    if (kShiftDst) {
+      const uint32_t before = static_cast<uint32_t>(d.addr) & 15u;
+      L.t = 16u - before;
+      wp -= before;
+      L.first = lane == 0;
+    }
+    // the first span goes to L2 now; each later one about a span before use
+    if (kPrefetch) prefetch_l2_lane0(lp, (left < kSpan ? left : kSpan) * kBlockBytes, lane);
+    lp += lane * 16;
+    wp += lane * 16;
 #pragma unroll
-  for (uint32_t u = 0; u < kStage; ++u)
-    cur[u] = u < nblk ? ld_unit(lp + u * kBlockBytes) : make_uint4(0u, 0u, 0u, 0u);
-  lp += kStageBytes;  // the next stage's loads
-
-  // This lane's unit of the next block, which is in cur[u].
-  auto unit = [&](uint32_t u) {
-    if (!kShiftSrc) return cur[u];
-    const uint4 y = shfl4(cur[u], (lane + 31) & 31u);
-    const uint4 before = select4(lane == 0, L.carry, y);
-    L.carry = y;
-    return take16(before, cur[u], L.t);
+    for (uint32_t u = 0; u < kStage; ++u)
+      cur[u] = u < left ? load(lp + u * kBlockBytes) : make_uint4(0u, 0u, 0u, 0u);
+    lp += kStageBytes;
   };
+  // Where the block in cur[u] was loaded, and this lane's unit of it.
+  auto place = [&](uint32_t u) { return lp + u * kBlockBytes - kStageBytes; };
+  auto unit = [&](uint32_t u) { return kShiftSrc ? take16(ld_unit_l1(place(u) - 16), cur[u], L.t) : cur[u]; };
   // One stage whose following stage is whole.
   auto stage = [&]() {
 #pragma unroll
     for (uint32_t u = 0; u < kStage; ++u) {
       if (Geo<MODE, SHIFT>::kLoadFirst) {
         const uint4 v = unit(u);
-        cur[u] = ld_unit(lp + u * kBlockBytes);
-        do_unit<MODE, DT, SHIFT>(L, v, wp + u * kBlockBytes, lb);
+        cur[u] = load(lp + u * kBlockBytes);
+        do_unit<MODE, DT, SHIFT>(L, v, place(u), wp + u * kBlockBytes, lb);
       } else {
-        do_unit<MODE, DT, SHIFT>(L, unit(u), wp + u * kBlockBytes, lb);
-        cur[u] = ld_unit(lp + u * kBlockBytes);
+        do_unit<MODE, DT, SHIFT>(L, unit(u), place(u), wp + u * kBlockBytes, lb);
+        cur[u] = load(lp + u * kBlockBytes);
       }
     }
     lp += kStageBytes;
     wp += kStageBytes;
   };
 
-  // Three loops cover a piece: (1) whole spans whose following stage is
-  // whole too, each span (one sum segment) a call-free loop of kSpan/kStage
-  // stages with no branch, preceded by the L2 prefetch of the next span and
-  // followed by its validity check -- the bulk of a long piece; (2) the
-  // stages left whose following stage is still whole, fewer than a span; (3)
-  // the last one or two stages, predicated.  Loop (2) keeps the predicated
-  // drain, which runs at about half the rate, to under 2 * kStage blocks.
-  uint32_t left = nblk;  // blocks not swept yet
-  while (left >= kSpan + kStage) {
-    if (kPrefetch && lane == 0) {
-      const uint32_t n = left - kSpan < kSpan ? left - kSpan : kSpan;
-      prefetch_l2(lp - kStageBytes + kSpanBytes, n * kBlockBytes);
+  if (n == 0) return;
+  begin();
+  for (;;) {
+    L.s[0] = L.s[1] = L.s[2] = L.s[3] = 0;
+    L.f = FpAcc{0ull, 0ull, 0ull, 0ull};
+    L.nonfinite = 0;
+    // Three loops cover a piece: (1) whole spans whose following stage is
+    // whole too, each span (one sum segment) a call-free loop of kSpan/kStage
+    // stages with no branch, preceded by the L2 prefetch of the next span and
+    // followed by its validity check -- the bulk of a long piece; (2) the
+    // stages left whose following stage is still whole, fewer than a span; (3)
+    // the last one or two stages, predicated.  Loop (2) keeps the predicated
+    // drain, which runs at about half the rate, to under 2 * kStage blocks.
+    while (left >= kSpan + kStage) {
+      if (kPrefetch && lane == 0) {
+        const uint32_t m = left - kSpan < kSpan ? left - kSpan : kSpan;
+        prefetch_l2(lp - kStageBytes + kSpanBytes, m * kBlockBytes);
+      }
+#pragma unroll 1
+      for (uint32_t st = 0; st < kSpan / kStage; ++st) stage();
+      if (kFp)
+        span_end<MODE, DT, kShiftSrc>(L, lp - kSpanBytes - kStageBytes - (kShiftSrc ? 16 - L.t : 0), kSpan, seg, lane);
+      ++seg;
+      left -= kSpan;
     }
+    if (kPrefetch && left > kSpan)
+      prefetch_l2_lane0(lp - kStageBytes + kSpanBytes, (left - kSpan) * kBlockBytes, lane);
+    uint32_t done = 0;  // blocks of the current span swept
 #pragma unroll 1
-    for (uint32_t st = 0; st < kSpan / kStage; ++st) stage();
-    if (kFp) span_end<MODE, DT, kShiftSrc>(L, lp - kSpanBytes - kStageBytes - (kShiftSrc ? 16 - L.t : 0), kSpan, seg, lane);
-    ++seg;
-    left -= kSpan;
-  }
-  if (kPrefetch && left > kSpan)
-    prefetch_l2_lane0(lp - kStageBytes + kSpanBytes, (left - kSpan) * kBlockBytes, lane);
-  uint32_t done = 0;  // blocks of the current span swept, whole stages
-#pragma unroll 1
-  for (; left >= 2 * kStage; left -= kStage, done += kStage) stage();
-  while (left > 0) {
+    for (; left >= 2 * kStage; left -= kStage, done += kStage) stage();
+    uint32_t m;  // blocks of the last stage
+    for (;;) {
 #pragma unroll
-    for (uint32_t u = 0; u < kStage; ++u) {
-      if (u < left) {
-        do_unit<MODE, DT, SHIFT>(L, unit(u), wp + u * kBlockBytes, lb);
-        if (kStage + u < left) cur[u] = ld_unit(lp + u * kBlockBytes);
+      for (uint32_t u = 0; u < kStage; ++u) {
+        if (u < left) {
+          do_unit<MODE, DT, SHIFT>(L, unit(u), place(u), wp + u * kBlockBytes, lb);
+          if (kStage + u < left) cur[u] = load(lp + u * kBlockBytes);
+        }
+      }
+      lp += kStageBytes;
+      wp += kStageBytes;
+      m = left < kStage ? left : kStage;
+      left -= m;
+      if (left == 0) break;
+      done += m;
+      if (done == kSpan) {
+        if (kFp)
+          span_end<MODE, DT, kShiftSrc>(L, lp - (kSpan + kStage) * kBlockBytes - (kShiftSrc ? 16 - L.t : 0), kSpan, seg,
+                                        lane);
+        ++seg;
+        done = 0;
       }
     }
-    lp += kStageBytes;
-    wp += kStageBytes;
-    const uint32_t n = left < kStage ? left : kStage;
-    left -= n;
-    if (kFp && (left == 0 || done + n == kSpan)) {
-      span_end<MODE, DT, kShiftSrc>(L, lp - (done + 2 * kStage) * kBlockBytes - (kShiftSrc ? 16 - L.t : 0), done + n, seg,
-                                    lane);
-      ++seg;
-      done = 0;
-    } else {
-      done += n;
-    }
-  }
+    // the open span (the piece's last): its first unit, blocks and slot
+    const uint8_t* sp = lp - (done + 2 * kStage) * kBlockBytes - (kShiftSrc ? 16 - L.t : 0);
+    double* last_seg = seg;
+    Record* rec = recs + r;
+    done += m;
+    // a shifted destination ends in the first granule after the blocks, m blocks
+    // into the last stage, with the end of the last unit
+    if (kShiftDst && lane == 0)
+      st_part<false>(wp - static_cast<int64_t>(kStage - m) * kBlockBytes,
+                     ld_unit_l1(lp - static_cast<int64_t>(2 * kStage - m) * kBlockBytes - 16), L.t);
+    ++r;
+    const bool more = --n > 0;
+    if (kFp) span_end<MODE, DT, kShiftSrc>(L, sp, done, last_seg, lane);
 
-  // A shifted destination ends in the first granule after the blocks.
-  if (kShiftDst && lane == 0) st_part<false>(dst - (16u - L.t) + static_cast<uint64_t>(nblk) * kBlockBytes, L.carry, L.t);
-
-  // ---- fold the 128 streams into the raw CRC of the piece
-  uint32_t v = mul_fold(0, L.s[0]) ^ L.s[1];
-  v = mul_fold(0, v) ^ L.s[2];
-  v = mul_fold(0, v) ^ L.s[3];
-  {
-    uint32_t o;
-    o = __shfl_down_sync(0xFFFFFFFFu, v, 1);
-    v = mul_fold(1, v) ^ o;
-    o = __shfl_down_sync(0xFFFFFFFFu, v, 2);
-    v = mul_fold(2, v) ^ o;
-    o = __shfl_down_sync(0xFFFFFFFFu, v, 4);
-    v = mul_fold(3, v) ^ o;
-    o = __shfl_down_sync(0xFFFFFFFFu, v, 8);
-    v = mul_fold(4, v) ^ o;
-    o = __shfl_down_sync(0xFFFFFFFFu, v, 16);
-    v = mul_fold(5, v) ^ o;
-  }
-
-  uint32_t nonfinite = L.nonfinite;
-  if (kFp) {
-#pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) nonfinite += __shfl_down_sync(0xFFFFFFFFu, nonfinite, m);
-  }
-  if (lane == 0) {
-    Record r;
-    r.crc = mul_fold(6, v);
-    r.nonfinite = nonfinite;
-    r.unused = 0.0;
-    *rec = r;
-  }
-}
-
-// A run of consecutive pieces of one class: a warp's own range, or a unit it
-// claimed.  A piece's descriptor says all its sweep needs, so a piece costs
-// one dependent load before its data, and the next one's is already in L1.
-// ALIGNED: every chunk of the class starts on a 16-byte boundary of its
-// tensor's memory; else none does.
-template <int MODE, int DT, bool ALIGNED>
-__device__ __forceinline__ void sweep_run(const SweepParams& p, uint32_t r, uint32_t n, uint32_t lane) {
-  for (; n > 0; --n, ++r) {
-    const PieceDesc d = p.pieces[r];
-    if (n > 1 && lane == 0) asm volatile("prefetch.global.L1 [%0];" ::"l"(p.pieces + r + 1));
-    uint8_t* tensor = reinterpret_cast<uint8_t*>(d.addr);
-    uint8_t* packed = (MODE == kModeFingerprint) ? nullptr : p.packed + d.payload_off;
-    sweep_piece<MODE, DT, !ALIGNED>(mode_unpacks(MODE) ? packed : tensor, mode_unpacks(MODE) ? tensor : packed, d.nblk,
-                                    lane, p.recs + r, p.segs + d.seg);
+    // ---- fold the 128 streams into the raw CRC of the piece
+    uint32_t v = mul_x32(L.s[0]) ^ L.s[1];
+    v = mul_x32(v) ^ L.s[2];
+    v = mul_x32(v) ^ L.s[3];
+    v = __reduce_xor_sync(0xFFFFFFFFu, mul_lane(v, lb));
+    const uint32_t nonfinite = kFp ? __reduce_add_sync(0xFFFFFFFFu, L.nonfinite) : 0u;
+    if (lane == 0) *rec = Record{v, nonfinite, 0.0};
+    if (!more) return;
+    begin();
   }
 }
 
@@ -803,19 +844,25 @@ __device__ __forceinline__ void sweep_run(const SweepParams& p, uint32_t r, uint
 // it runs every element type as bytes.)
 template <int MODE>
 __device__ __forceinline__ void sweep_class(const SweepParams& p, const RunDesc& rd, uint32_t lane) {
+  // a piece's descriptor says all its sweep needs: one dependent load, and the
+  // next one's is on its way to L1
+  auto get = [&](uint32_t r, bool more) {
+    if (more && lane == 0) asm volatile("prefetch.global.L1 [%0];" ::"l"(p.pieces + r + 1));
+    return p.pieces[r];
+  };
   if constexpr (!mode_sums(MODE)) {
     if (rd.cls & 1u)
-      sweep_run<MODE, kDtBytes, true>(p, rd.first, rd.n, lane);
+      sweep_run<MODE, kDtBytes, false>(p.packed, p.segs, p.recs, get, rd.first, rd.n, lane);
     else
-      sweep_run<MODE, kDtBytes, false>(p, rd.first, rd.n, lane);
+      sweep_run<MODE, kDtBytes, true>(p.packed, p.segs, p.recs, get, rd.first, rd.n, lane);
   } else {
     switch (rd.cls) {
-      case kDtF32 * 2 + 1: sweep_run<MODE, kDtF32, true>(p, rd.first, rd.n, lane); break;
-      case kDtBf16 * 2 + 1: sweep_run<MODE, kDtBf16, true>(p, rd.first, rd.n, lane); break;
-      case kDtBytes * 2 + 1: sweep_run<MODE, kDtBytes, true>(p, rd.first, rd.n, lane); break;
-      case kDtF32 * 2: sweep_run<MODE, kDtF32, false>(p, rd.first, rd.n, lane); break;
-      case kDtBf16 * 2: sweep_run<MODE, kDtBf16, false>(p, rd.first, rd.n, lane); break;
-      default: sweep_run<MODE, kDtBytes, false>(p, rd.first, rd.n, lane); break;
+      case kDtF32 * 2 + 1: sweep_run<MODE, kDtF32, false>(p.packed, p.segs, p.recs, get, rd.first, rd.n, lane); break;
+      case kDtBf16 * 2 + 1: sweep_run<MODE, kDtBf16, false>(p.packed, p.segs, p.recs, get, rd.first, rd.n, lane); break;
+      case kDtBytes * 2 + 1: sweep_run<MODE, kDtBytes, false>(p.packed, p.segs, p.recs, get, rd.first, rd.n, lane); break;
+      case kDtF32 * 2: sweep_run<MODE, kDtF32, true>(p.packed, p.segs, p.recs, get, rd.first, rd.n, lane); break;
+      case kDtBf16 * 2: sweep_run<MODE, kDtBf16, true>(p.packed, p.segs, p.recs, get, rd.first, rd.n, lane); break;
+      default: sweep_run<MODE, kDtBytes, true>(p.packed, p.segs, p.recs, get, rd.first, rd.n, lane); break;
     }
   }
 }
@@ -827,6 +874,15 @@ __device__ __forceinline__ void sweep_class(const SweepParams& p, const RunDesc&
 // 10 us for its 32 KiB) costs its launch more than the tail (GPT-2 small: its
 // SMs end between 270 and 282 us without units, all at 295 with 8% in units).
 __host__ __device__ constexpr bool mode_claims(int m) { return m != kModeFingerprint; }
+
+// The CTA's shared memory: braid tables, lane table.
+template <int MODE>
+__device__ __forceinline__ void fill_smem() {
+  start_lane_fold<Cta<MODE>::kThreads>();
+  fill_tables<Cta<MODE>::kThreads>();
+  finish_lane_fold();
+  __syncthreads();
+}
 
 // Every class of a batch in one launch: each warp sweeps a run of its own
 // class, and the plan spreads each class's warps over all CTAs, so warps that
@@ -844,8 +900,7 @@ __host__ __device__ constexpr bool mode_claims(int m) { return m != kModeFingerp
 // small's unpack lost 4%.)
 template <int MODE>
 __global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) sweep_kernel(SweepParams p) {
-  fill_tables<Cta<MODE>::kThreads>();
-  __syncthreads();
+  fill_smem<MODE>();
   const uint32_t lane = threadIdx.x & 31u;
   RunDesc rd = p.warps[blockIdx.x * Cta<MODE>::kWarps + (threadIdx.x >> 5)];
   for (;;) {
@@ -863,37 +918,38 @@ __global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) sweep_kernel(SweepPara
 // ids[w] into recs[w].  Every variant is a separate function, so this cold
 // kernel's dispatch does not burden the registers of the hot ones.
 template <int MODE, int DT, bool ALIGNED>
-__device__ __noinline__ void list_piece(uint8_t* tensor, uint8_t* packed, uint32_t n, uint32_t lane, Record* rec,
-                                        double* segs) {
-  sweep_piece<MODE, DT, !ALIGNED>(mode_unpacks(MODE) ? packed : tensor, mode_unpacks(MODE) ? tensor : packed, n, lane,
-                                  rec, segs);
+__device__ __noinline__ void list_piece(const ListParams& p, uint64_t w, uint32_t lane) {
+  auto get = [&](uint32_t, bool) {
+    const ChunkDesc cd = p.chunks[p.ids[w]];
+    PieceDesc d;
+    d.addr = cd.addr;
+    d.payload_off = cd.payload_off;
+    d.seg = cd.seg_base;
+    d.nblk = static_cast<uint32_t>(cd.len / kBlockBytes);
+    return d;
+  };
+  sweep_run<MODE, DT, !ALIGNED>(p.packed, p.segs, p.recs + w, get, 0, 1, lane);
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) list_kernel(ListParams p) {
-  fill_tables<Cta<MODE>::kThreads>();
-  __syncthreads();
+__global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) list_kernel(const __grid_constant__ ListParams p) {
+  fill_smem<MODE>();
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t w = static_cast<uint64_t>(blockIdx.x) * Cta<MODE>::kWarps + (threadIdx.x >> 5);
   if (w >= p.n) return;
   const ChunkDesc cd = p.chunks[p.ids[w]];
-  const uint32_t nb = static_cast<uint32_t>(cd.len / kBlockBytes);
-  if (nb == 0) return;
-  uint8_t* tensor = reinterpret_cast<uint8_t*>(cd.addr);
-  uint8_t* packed = p.packed + cd.payload_off;
+  if (cd.len < static_cast<uint64_t>(kBlockBytes)) return;
   const bool aligned = (cd.sweep_class & 1u) != 0;
   const uint32_t dt = mode_sums(MODE) ? cd.dtype : kDtBytes;
-  double* segs = p.segs + cd.seg_base;
-  Record* rec = p.recs + w;
   if (dt == kDtF32) {
-    if (aligned) list_piece<MODE, kDtF32, true>(tensor, packed, nb, lane, rec, segs);
-    else list_piece<MODE, kDtF32, false>(tensor, packed, nb, lane, rec, segs);
+    if (aligned) list_piece<MODE, kDtF32, true>(p, w, lane);
+    else list_piece<MODE, kDtF32, false>(p, w, lane);
   } else if (dt == kDtBf16) {
-    if (aligned) list_piece<MODE, kDtBf16, true>(tensor, packed, nb, lane, rec, segs);
-    else list_piece<MODE, kDtBf16, false>(tensor, packed, nb, lane, rec, segs);
+    if (aligned) list_piece<MODE, kDtBf16, true>(p, w, lane);
+    else list_piece<MODE, kDtBf16, false>(p, w, lane);
   } else {
-    if (aligned) list_piece<MODE, kDtBytes, true>(tensor, packed, nb, lane, rec, segs);
-    else list_piece<MODE, kDtBytes, false>(tensor, packed, nb, lane, rec, segs);
+    if (aligned) list_piece<MODE, kDtBytes, true>(p, w, lane);
+    else list_piece<MODE, kDtBytes, false>(p, w, lane);
   }
 }
 
@@ -901,7 +957,7 @@ template <int MODE>
 cudaError_t launch_list(const ListParams& p, cudaStream_t s) {
   if (p.n == 0) return cudaSuccess;
   const uint64_t ctas = (p.n + Cta<MODE>::kWarps - 1) / Cta<MODE>::kWarps;
-  list_kernel<MODE><<<static_cast<unsigned>(ctas), Cta<MODE>::kThreads, kTableBytes, s>>>(p);
+  list_kernel<MODE><<<static_cast<unsigned>(ctas), Cta<MODE>::kThreads, kSweepSmem, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -910,17 +966,17 @@ cudaError_t launch_list(const ListParams& p, cudaStream_t s) {
 // Opt the kernels of one mode in to their shared-memory size; launch them.
 template <int MODE>
 cudaError_t configure_mode() {
-  cudaError_t e = cudaFuncSetAttribute(sweep_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
+  cudaError_t e = cudaFuncSetAttribute(sweep_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
   if constexpr (MODE != kModeFingerprint) {  // no call fingerprints a list
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(list_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
+      e = cudaFuncSetAttribute(list_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
   }
   return e;
 }
 
 template <int MODE>
 cudaError_t launch_mode(const SweepParams& p, int n_ctas, cudaStream_t s) {
-  sweep_kernel<MODE><<<n_ctas, Cta<MODE>::kThreads, kTableBytes, s>>>(p);
+  sweep_kernel<MODE><<<n_ctas, Cta<MODE>::kThreads, kSweepSmem, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -4,7 +4,7 @@
 //
 // A warp sweeps a range of one class only.  The classes are not equally
 // costly per block: a bf16 block holds twice the elements of an fp32 block,
-// so the fingerprint spends about a third more instructions on it, while
+// so the fingerprint spends almost half as much again on it, while
 // pack and unpack are bound by memory in every class.  The warps are shared
 // in proportion to each class's blocks times its weight (percent of an fp32
 // block), so that the classes' warps finish together; each class's warps are
@@ -17,19 +17,19 @@
 #include "layout.h"
 
 #ifndef FR_MIX_W_BF16
-// Fingerprint: a bf16 block costs 1.35 fp32 blocks.  Measured, GPT-2 small
-// (1.7 GB) / Llama-8B shard (14 GB) in us: 1.25 306 / 2116, 1.30 309 / 2111,
-// 1.35 292 / 2116, 1.40 293 / 2127.
-#define FR_MIX_W_BF16 135
+// Fingerprint: a bf16 block costs 1.45 fp32 blocks.  Measured, GPT-2 small
+// (1.7 GB) / Llama-8B shard (14 GB) in us: 1.35 293 / 2085, 1.40 289 / 2079,
+// 1.45 283 / 2092, 1.50 283 / 2103.
+#define FR_MIX_W_BF16 145
 #endif
 #ifndef FR_MIX_W_BF16_PACK
 #define FR_MIX_W_BF16_PACK 100  // pack and unpack: memory-bound, all blocks alike
 #endif
-// Fingerprint: a block of a chunk off the 16-byte boundary costs 0.4 fp32
-// blocks more (0.2 / 0.4 / 0.6: 607 / 597 / 603 us for 2.5 GB of views); pack
+// Fingerprint: a block of a chunk off the 16-byte boundary costs 0.25 fp32
+// blocks more (0.15 / 0.25 / 0.4: 539 / 529 / 560 us for 2.5 GB of views); pack
 // and unpack even it out with their units.
 #ifndef FR_MIX_W_SHIFT
-#define FR_MIX_W_SHIFT 40
+#define FR_MIX_W_SHIFT 25
 #endif
 #ifndef FR_MIX_W_BYTES
 #define FR_MIX_W_BYTES 100

@@ -110,6 +110,17 @@ int main() {
         for (uint64_t dyn : {0ull, 8ull, 50ull})
           if (check(lens, Wq, dyn, 1 + next(4))) return 1;
     }
+  // units: all of the claimed segments, never growing, single ones at the end
+  for (uint64_t n : {1ull, 5ull, 152ull, 3041ull, 20000ull, 155000ull, 2000000ull})
+    for (uint64_t Wq : {1ull, 40ull, 1520ull, 3040ull}) {
+      uint64_t left = n, before = FR_UNIT_MAX;
+      while (left > 0) {
+        const uint64_t u = unit_segs(left, Wq);
+        EXPECT(u >= 1 && u <= left && u <= before && (left > Wq || u == 1));
+        before = u;
+        left -= u;
+      }
+    }
   if (check({}, 5, 0, 1) || check({100, 511, 0}, 5, 8, 2)) return 1;
   std::printf("seg_walk ok\n");
   return 0;

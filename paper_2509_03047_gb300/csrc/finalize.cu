@@ -205,6 +205,7 @@ __global__ void __launch_bounds__(kFinThreads, FR_FIN_MINB) finalize_kernel(Fina
     for (int i = 0; i < kLaneMulWords / 4 / kFinThreads; ++i) dst[threadIdx.x + i * kFinThreads] = src[threadIdx.x + i * kFinThreads];
   }
   __syncthreads();
+  wait_for_kernel_before();
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t* LM = lm_s.t + lane;
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * kFinWarps;
@@ -575,6 +576,7 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(Pred pred, uin
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t lt = (1u << lane) - 1u;  // lanes below this one
   uint64_t base = 0;
+  wait_for_kernel_before();
   if (tid == 0) pred.prefetch(0, n < kTile ? n : kTile);
   for (uint64_t t0 = 0; t0 < n; t0 += kTile) {
     // the next tile streams into L2 while this one is tested
@@ -650,6 +652,7 @@ __global__ void __cluster_dims__(kCompactCluster, 1, 1) __launch_bounds__(kCompa
   const uint64_t rounds = (n_tiles + kCompactCluster - 1) / kCompactCluster;
   constexpr uint64_t kStride = static_cast<uint64_t>(kCompactCluster) * kTile;
   uint64_t base = 0;
+  wait_for_kernel_before();
   if (tid == 0 && static_cast<uint64_t>(rank) * kTile < n) {
     const uint64_t t0 = static_cast<uint64_t>(rank) * kTile;
     pred.prefetch(t0, n - t0 < kTile ? n - t0 : kTile);
@@ -715,10 +718,8 @@ template <class Pred>
 cudaError_t launch_compact(const Pred& pred, uint64_t n, uint32_t* out, uint64_t cap, uint64_t* count,
                            uint32_t* status, cudaStream_t s) {
   if (n > static_cast<uint64_t>(kTile))
-    compact_cluster_kernel<Pred><<<kCompactCluster, kCompactThreads, 0, s>>>(pred, n, out, cap, count, status);
-  else
-    compact_kernel<Pred><<<1, kCompactThreads, 0, s>>>(pred, n, out, cap, count, status);
-  return cudaGetLastError();
+    return launch_chained(compact_cluster_kernel<Pred>, kCompactCluster, kCompactThreads, 0, s, pred, n, out, cap, count, status);
+  return launch_chained(compact_kernel<Pred>, 1, kCompactThreads, 0, s, pred, n, out, cap, count, status);
 }
 
 }  // namespace
@@ -735,15 +736,10 @@ cudaError_t launch_finalize(int mode, const FinalizeParams& p, cudaStream_t s) {
   const uint64_t cap = static_cast<uint64_t>(n_sm > 0 ? n_sm : 1) * FR_FIN_MINB;
   const uint64_t want = (p.c_end - p.c_begin + kFinWarps - 1) / kFinWarps;
   const int grid = static_cast<int>(want < cap ? want : cap);
-  if (mode == kModeFingerprint)
-    finalize_kernel<kModeFingerprint><<<grid, kFinThreads, 0, s>>>(p);
-  else if (mode == kModePack)
-    finalize_kernel<kModePack><<<grid, kFinThreads, 0, s>>>(p);
-  else if (mode == kModeUnpackFp)
-    finalize_kernel<kModeUnpackFp><<<grid, kFinThreads, 0, s>>>(p);
-  else
-    finalize_kernel<kModeUnpack><<<grid, kFinThreads, 0, s>>>(p);
-  return cudaGetLastError();
+  if (mode == kModeFingerprint) return launch_chained(finalize_kernel<kModeFingerprint>, grid, kFinThreads, 0, s, p);
+  if (mode == kModePack) return launch_chained(finalize_kernel<kModePack>, grid, kFinThreads, 0, s, p);
+  if (mode == kModeUnpackFp) return launch_chained(finalize_kernel<kModeUnpackFp>, grid, kFinThreads, 0, s, p);
+  return launch_chained(finalize_kernel<kModeUnpack>, grid, kFinThreads, 0, s, p);
 }
 
 cudaError_t launch_compact_flags(const uint8_t* flags, uint64_t n, uint32_t* out, uint64_t cap,

@@ -189,12 +189,16 @@ class PlanMemory {
     places_.push_back({reinterpret_cast<void**>(at), scratch_, true});
     scratch_ = align_up(scratch_ + count * sizeof(T), kAlign);
   }
-  // Allocates, copies the tables and sets every pointer.
+  // Allocates, copies the tables and sets every pointer.  The wait is for the
+  // copy's last part: one from pageable memory may return while that is still
+  // on its way, on the legacy stream, and a call on a non-blocking stream is
+  // not ordered after it.
   cudaError_t commit(void** memory) {
     const uint64_t first = align_up(tables_.size(), kAlign);
     cudaError_t e = cudaMalloc(memory, std::max<uint64_t>(first + scratch_, kAlign));
     if (e != cudaSuccess) return e;
     if (!tables_.empty()) e = cudaMemcpy(*memory, tables_.data(), tables_.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     for (const Place& q : places_) *q.at = static_cast<uint8_t*>(*memory) + (q.scratch ? first : 0) + q.off;
     return e;
   }

@@ -118,7 +118,7 @@ __host__ __device__ constexpr PowTables make_pow_tables() {
 
 // x^(8n) mod P on the host, from the per-byte power tables.
 inline uint32_t host_xpow8(uint64_t n) {
-  static const PowTables T = make_pow_tables();
+  static constexpr PowTables T = make_pow_tables();
   uint32_t r = kOne;
   for (int k = 0; n != 0; ++k, n >>= 8)
     if (n & 255u) r = r == kOne ? T.p[k][n & 255u] : gf_mulmod(r, T.p[k][n & 255u]);
@@ -126,42 +126,45 @@ inline uint32_t host_xpow8(uint64_t n) {
 }
 
 // Tables over 12-bit digits for what a plan computes once per chunk or piece:
-// digit i of `low` is start * x^(8 unit i), of `high` x^(8 unit 4096 i), so a
+// digit i of `low` is START * x^(8 UNIT i), of `high` x^(8 UNIT 4096 i), so a
 // count under 4096 units takes no multiplication and one under 2^24 takes one.
 // (From per-byte powers it was two to four, 40 ns each: 1.3 of the 2.6 ms that
-// a plan over 8 tensors in 8 batches took.)
+// a plan over 8 tensors in 8 batches took.)  Constants of the program, 32 KiB
+// each: filled on first use they made a process's first plan 0.8 ms longer (a 15
+// MB state's, host side alone on an x86 core: first 1.2-1.9 -> 0.5-0.7 ms, later
+// ones 0.27 either way).
 struct DigitTables {
   uint32_t low[4096], high[4096];
-  uint64_t unit;
-  DigitTables(uint32_t start, uint64_t unit_bytes) : unit(unit_bytes) {
-    const uint32_t one = gf_xpow(8 * unit), big = gf_xpow(8 * unit * 4096);
-    low[0] = start;
-    high[0] = kOne;
-    for (int i = 1; i < 4096; ++i) {
-      low[i] = gf_mulmod(low[i - 1], one);
-      high[i] = gf_mulmod(high[i - 1], big);
-    }
+};
+constexpr DigitTables make_digit_tables(uint32_t start, uint64_t unit) {
+  DigitTables out{};
+  const uint32_t one = gf_xpow(8 * unit), big = gf_xpow(8 * unit * 4096);
+  out.low[0] = start;
+  out.high[0] = kOne;
+  for (int i = 1; i < 4096; ++i) {
+    out.low[i] = gf_mulmod(out.low[i - 1], one);
+    out.high[i] = gf_mulmod(out.high[i - 1], big);
   }
-  // start * x^(8 unit n) mod P
-  uint32_t at(uint64_t n) const {
-    uint32_t r = low[n & 4095u];
-    if ((n >> 12) & 4095u) r = gf_mulmod(r, high[(n >> 12) & 4095u]);
-    if (n >> 24) r = gf_mulmod(r, host_xpow8((n >> 24 << 24) * unit));
+  return out;
+}
+// (A template, so that only the files that use a table evaluate it.)
+template <uint32_t START, uint64_t UNIT>
+struct Digits {
+  static constexpr DigitTables T = make_digit_tables(START, UNIT);
+  // START * x^(8 UNIT n) mod P, UNIT n < 2^48
+  static uint32_t at(uint64_t n) {
+    uint32_t r = T.low[n & 4095u];
+    if ((n >> 12) & 4095u) r = gf_mulmod(r, T.high[(n >> 12) & 4095u]);
+    if (n >> 24) r = gf_mulmod(r, host_xpow8((n >> 24 << 24) * UNIT));
     return r;
   }
 };
 
 // The CRC-32C preset and final XOR of an n-byte message as one term:
 // crc = raw ^ crc_xor_term(n), raw being the CRC register run from zero.
-inline uint32_t host_crc_xor_term(uint64_t n) {
-  static const DigitTables T(0xFFFFFFFFu, 1);
-  return T.at(n) ^ 0xFFFFFFFFu;
-}
+inline uint32_t host_crc_xor_term(uint64_t n) { return Digits<0xFFFFFFFFu, 1>::at(n) ^ 0xFFFFFFFFu; }
 
 // x^(8n) mod P for n = `blocks` 512-byte blocks.
-inline uint32_t host_xpow8_blocks(uint64_t blocks) {
-  static const DigitTables T(kOne, kBlockBytes);
-  return T.at(blocks);
-}
+inline uint32_t host_xpow8_blocks(uint64_t blocks) { return Digits<kOne, kBlockBytes>::at(blocks); }
 
 }  // namespace frk

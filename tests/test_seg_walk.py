@@ -49,3 +49,14 @@ def test_crc_xor_term(tmp_path, orc):
         '  std::printf("%%08x\\n", frk::host_crc_xor_term(%dull));\n' % n for n in sizes) + "}\n")
     got = [int(v, 16) for v in _run(tmp_path, str(src)).split()]
     assert got == [orc.crc32c(np.zeros(n, dtype=np.uint8)) for n in sizes]
+
+
+def test_power_tables_are_constants_of_the_program(tmp_path):
+    """No call fills a table: a process's first plan takes what a later one takes."""
+    src = tmp_path / "t.cc"
+    src.write_text('#include <cstdio>\n#include "gf2.cuh"\nusing namespace frk;\nint main() {\n' + "".join(
+        "  { constexpr const DigitTables& T = Digits<%s, %d>::T;\n"
+        "    static_assert(T.low[4095] == gf_mulmod(%s, gf_xpow(8ull * %d * 4095)), \"low\");\n"
+        "    static_assert(T.high[4095] == gf_xpow(8ull * %d * 4096 * 4095), \"high\"); }\n" % (s, u, s, u, u)
+        for s, u in (("0xFFFFFFFFu", 1), ("kOne", 512))) + '  std::puts("ok");\n}\n')
+    assert _run(tmp_path, str(src)) == "ok\n"

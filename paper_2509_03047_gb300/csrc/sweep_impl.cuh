@@ -484,24 +484,27 @@ __device__ __noinline__ Exact slow_span(const uint8_t* sp, uint32_t n) {
 }
 
 // The same for lane l's units, in every lane: lane k loads the unit of block
-// k, and all lanes add the words in the order slow_span does, taking them from
-// lane k by shuffle.  One lane that needs the fallback (one NaN) is the common
-// case, and its warp may be all that a launch still waits for: this way it
-// waits for one load, not for 32 in turn.  GB300, a 15 MB state with 3 NaNs
+// k (of 32 at a time), and all lanes add the words in the order slow_span does,
+// taking them from lane k by shuffle.  One lane that needs the fallback (one
+// NaN) is the common case, and its warp may be all that a launch still waits
+// for: this way it waits for one load, not for 32 in turn.  GB300, a 15 MB state with 3 NaNs
 // (L2-resident, as a graph), us: fingerprint 24.5 -> 17.3, pack 24.7 -> 16.9;
 // without NaN 15.2.
 template <int DT, bool SHIFT>
 __device__ __noinline__ Exact slow_span_by_warp(const uint8_t* sp, uint32_t n, uint32_t l, uint32_t lane) {
   const uint8_t* first = sp + (static_cast<int32_t>(l) - static_cast<int32_t>(lane)) * 16;  // lane l's first unit
-  uint4 v = make_uint4(0u, 0u, 0u, 0u);
-  if (lane < n) v = ld_unit_at<SHIFT>(first + lane * kBlockBytes);
   ExactSum x;
 #pragma unroll 1
-  for (uint32_t k = 0; k < n; ++k) {
-    x.add_word<DT>(__shfl_sync(0xFFFFFFFFu, v.x, k));
-    x.add_word<DT>(__shfl_sync(0xFFFFFFFFu, v.y, k));
-    x.add_word<DT>(__shfl_sync(0xFFFFFFFFu, v.z, k));
-    x.add_word<DT>(__shfl_sync(0xFFFFFFFFu, v.w, k));
+  for (uint32_t g = 0; g < kSpan; g += 32) {  // (one pass unless a segment is built larger)
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (g + lane < n) v = ld_unit_at<SHIFT>(first + (g + lane) * kBlockBytes);
+#pragma unroll 1
+    for (uint32_t k = g; k < n && (kSpan <= 32 || k < g + 32); ++k) {
+      x.add_word<DT>(__shfl_sync(0xFFFFFFFFu, v.x, k - g));
+      x.add_word<DT>(__shfl_sync(0xFFFFFFFFu, v.y, k - g));
+      x.add_word<DT>(__shfl_sync(0xFFFFFFFFu, v.z, k - g));
+      x.add_word<DT>(__shfl_sync(0xFFFFFFFFu, v.w, k - g));
+    }
   }
   const double d = x.odd ? odd_squares<DT, SHIFT>(first, n) : 0.0;
   return Exact{(static_cast<double>(x.hi) + static_cast<double>(x.lo)) + d, x.nonfinite};

@@ -72,9 +72,13 @@ constexpr int kTableBytes = 4 * 256 * 32 * 4;  // 4 tables x 256 entries x 32 la
 #endif
 // Up to this many lanes of a segment that need the exact fallback take it in
 // turn by the whole warp (slow_span_by_warp), more take it side by side
-// (slow_span).
+// (slow_span).  In turn, each lane costs 3.5 us more; side by side they cost the
+// same together however many.  Measured, fingerprint of 15 MB of fp32 as a
+// graph, us, in turn / side by side, NaN lanes in one segment: 1 lane 17 / 25, 2
+// lanes 20 / 25, 3 lanes 24 / 25, 4 lanes 27 / 25; in every segment: 22 / 27, 30 /
+// 27, 37 / 27, 44 / 27.
 #ifndef FR_SLOW_WARP_LANES
-#define FR_SLOW_WARP_LANES 4
+#define FR_SLOW_WARP_LANES 2
 #endif
 #ifndef FR_STAGE_PACK
 #define FR_STAGE_PACK 4

@@ -1,8 +1,8 @@
 """GPU tests of the sum segments that are redone exactly: by the whole warp for
-up to 4 of its lanes, lane by lane beyond that.
+up to 2 of its lanes, lane by lane beyond that.
 
 A lane owns bytes 16l..16l+15 of every 512-byte block.  NaN and infinities put
-into 1, 4, 5 and 32 lanes of one segment take both ways, with elements whose
+into 1 to 5 and 32 lanes of one segment take both ways, with elements whose
 squares under- or overflow fp32 among them (added in fp64) and in a segment cut
 short; counts must equal the oracle's and sums agree to 1e-9."""
 import os
@@ -21,7 +21,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 @pytest.mark.parametrize("shift", [0, 4])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
-@pytest.mark.parametrize("lanes", [1, 4, 5, 32])
+@pytest.mark.parametrize("lanes", [1, 2, 3, 4, 5, 32])
 def test_segments_redone_exactly(dtype, lanes, shift):
     gen = torch.Generator(device="cuda").manual_seed(lanes)
     per_lane = 16 // dtype.itemsize

@@ -223,9 +223,8 @@ void free_device(fr_plan p) {
 
 // Cut the chunks [bounds[b], bounds[b+1]) of every batch b into sweep work for
 // `n_ctas` CTAs: per batch and class, the class's 16 KiB segments in chunk
-// order are split into runs of equal estimated cost (the rule of
-// split_ranges), one per warp, and every (warp, chunk) overlap is a piece with
-// a record.  Records are numbered batch by batch, class by class, so each
+// order are split into runs of equal estimated cost (SegWalk::to_cost), one per
+// warp, and every (warp, chunk) overlap is a piece with a record.  Records are numbered batch by batch, class by class, so each
 // chunk's records are consecutive.  `min_recs`: record slots to allocate at
 // least (list-mode calls use one slot per listed chunk).
 // The classes of a batch share the warps in proportion to their weighted

@@ -189,7 +189,7 @@ __device__ const LaneFoldTable g_lane_fold = make_lane_fold_table();
 constexpr int kSweepSmem = kTableBytes + kLaneFoldWords * 4;
 
 // Starts this thread's share of the lane table on its way to shared memory;
-// fill_tables waits for it.
+// finish_lane_fold waits for it.
 template <int kThreads>
 __device__ __forceinline__ void start_lane_fold() {
   const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(g_smem + kTableBytes));

@@ -7,9 +7,11 @@
 // so the fingerprint spends almost half as much again on it, while
 // pack and unpack are bound by memory in every class.  The warps are shared
 // in proportion to each class's blocks times its weight (percent of an fp32
-// block), so that the classes' warps finish together; each class's warps are
-// spread round-robin over the CTAs, so every SM runs a mix.  Within a class
-// the ranges are cut by an estimated cost per segment (split_ranges).
+// block), so that the classes' warps finish together.  The classes of shifted
+// chunks take the launch's first warps, those of aligned chunks the others,
+// and within either range each class's warps are spread round-robin over the
+// CTAs, so an SM runs a mix of element types (place_warps).  Within a class the
+// ranges are cut by an estimated cost per segment (seg_cost, SegWalk::to_cost).
 #pragma once
 
 #include <cstdint>
@@ -19,7 +21,8 @@
 #ifndef FR_MIX_W_BF16
 // Fingerprint: a bf16 block costs 1.45 fp32 blocks.  Measured, GPT-2 small
 // (1.7 GB) / Llama-8B shard (14 GB) in us: 1.35 293 / 2085, 1.40 289 / 2079,
-// 1.45 283 / 2092, 1.50 283 / 2103.
+// 1.45 283 / 2092, 1.50 283 / 2103.  A compromise: the shard alone is best at
+// 1.40, by 0.6%, GPT-2 small at 1.45, by 2%.
 #define FR_MIX_W_BF16 145
 #endif
 #ifndef FR_MIX_W_BF16_PACK
@@ -54,26 +57,35 @@
 #endif
 
 // A pack or unpack launch keeps FR_DYN_PCT percent of each class's segments
-// out of the warps' own runs, as units of at most FR_UNIT_SEGS segments that
-// warps claim at run time, when the class has at least FR_CLAIM_MIN segments
-// per warp.  Measured on GB300, pack / unpack of GPT-2 small: no units 562 /
-// 564 us; 8% in units of 1, 2 and 4 segments 547 / 538, 545 / 538, 549 / 540;
-// 4% of 1 553 / 548.
+// out of the warps' own runs, as units that warps claim at run time, of
+// FR_UNIT_SEGS segments or a few more (unit_segs).  Measured on GB300, pack /
+// unpack of GPT-2 small: no units 562 / 564 us; 8% in units of 1, 2 and 4
+// segments 547 / 538, 545 / 538, 549 / 540; 4% of 1 553 / 548.
 #ifndef FR_DYN_PCT
 #define FR_DYN_PCT 8
 #endif
 #ifndef FR_UNIT_SEGS
 #define FR_UNIT_SEGS 2
 #endif
-// A large state starts with larger units, up to FR_UNIT_MAX segments: with 32
-// KiB ones the last 8% of a 32 GB state was 77,000 records, 512 for a 16 MiB
-// chunk (its pack 10,179 us, 10,155 with larger ones; smaller states equal).
+// A large state starts with larger units, 1 / FR_UNIT_SHARE of a warp's share of
+// what is left but at most FR_UNIT_MAX segments (256 KiB): with 32 KiB ones the
+// last 8% of a 32 GB state was 77,000 records, 512 for a 16 MiB chunk (its pack
+// 10,179 us, 10,155 with larger ones; smaller states equal).  The two values
+// matter little: pack of 32 GB with a share of 1, 2, 4, 8, 16: 10,140 / 10,148 /
+// 10,152 / 10,153 / 10,160 us, with a maximum of 2, 16, 64: 10,161 / 10,152 /
+// 10,154; GPT-2 small, the Llama-8B shard and the fragmented states move by 0.2%.
 #ifndef FR_UNIT_SHARE
 #define FR_UNIT_SHARE 4
 #endif
 #ifndef FR_UNIT_MAX
 #define FR_UNIT_MAX 16
 #endif
+// A class has units only from FR_CLAIM_MIN segments per warp on.  Measured, no
+// units / units, us, by segments per warp: pack of 130 MB (2.6) 50.0 / 49.6, 159
+// MB (3.2) 61.5 / 59.9, 203 MB (4.1) 76.2 / 73.0, 300 MB (5.9) 107 / 102; GPT-2
+// small restored in 32 batches (2.2) 1,650 / 1,665, in 24 (2.9) 1,474 / 1,485, in
+// 16 (4.4) 1,470 / 1,461.  With 4 no batched restore loses and a state of 3 to 4
+// segments per warp forgoes 2%.
 #ifndef FR_CLAIM_MIN
 #define FR_CLAIM_MIN 4
 #endif
@@ -128,23 +140,6 @@ inline uint64_t seg_cost(uint64_t blocks, bool first) {
   return FR_SPLIT_BLK * blocks + FR_SPLIT_SEG + (first ? FR_SPLIT_PIECE : 0);
 }
 
-// bnd[w], w = 0..Wq: the segment where warp w's range starts, given the cost
-// prefix cost(s) of segments [0, s) for s = 0..n (nondecreasing): the last
-// boundary whose prefix is at most w / Wq of the total (bnd[0] = 0 even if
-// the first segments cost nothing, bnd[Wq] = n).  With unit costs this is
-// floor(n * w / Wq).
-template <class Prefix>
-inline void split_ranges(const Prefix& cost, uint64_t n, uint64_t Wq, uint64_t* bnd) {
-  const unsigned __int128 total = cost(n);
-  uint64_t s = 0;
-  bnd[0] = 0;
-  for (uint64_t w = 1; w <= Wq; ++w) {
-    const unsigned __int128 target = total * w;
-    while (s < n && static_cast<unsigned __int128>(cost(s + 1)) * Wq <= target) ++s;
-    bnd[w] = s;
-  }
-}
-
 // How many of the last segments of a class of n, shared by Wq warps, are cut
 // into units (none for the fingerprint, see mode_claims, nor while the warps
 // have too few segments each for a tail to even out).
@@ -178,14 +173,6 @@ inline void spread_range(const uint64_t* wc, const int* qs, int m, uint64_t firs
       if (++cta * wpc >= end) cta = first / wpc, ++row;
     }
   }
-}
-
-// The same for n <= kClassCount classes over a whole launch of W warps.
-inline void spread_warps(const uint64_t* wc, int n, uint64_t W, int, int warps_per_cta, uint32_t* slot,
-                         uint64_t stride) {
-  int qs[kClassCount];
-  for (int q = 0; q < n; ++q) qs[q] = q;
-  spread_range(wc, qs, n, 0, W, warps_per_cta, slot, stride);
 }
 
 // The warps of a launch's classes (class q is sweep class cls[q]): those of

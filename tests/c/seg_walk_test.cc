@@ -1,11 +1,12 @@
 // seg_walk_test.cc -- checks the planner's segment walk (csrc/seg_walk.h)
 // against the plain rule it stands for: split_ranges over the prefix sums of
-// every segment's cost (csrc/warp_share.h).  Exits 0 and prints "seg_walk ok".
+// every segment's cost (split_ranges.h).  Exits 0 and prints "seg_walk ok".
 #include <cstdio>
 #include <cstring>
 #include <vector>
 
 #include "seg_walk.h"
+#include "split_ranges.h"
 
 using namespace frk;
 

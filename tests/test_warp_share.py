@@ -1,8 +1,10 @@
 """The host rule that shares one sweep launch's warps among the element-type /
 alignment classes (csrc/warp_share.h), compiled with the host C++ compiler
 and checked by tests/c/warp_share_test.cc: warp counts sum to the launch,
-follow the weighted block counts, give every class at least one warp, and
-every CTA gets an even share of every class; within a class the ranges are
+follow the weighted block counts and give every class at least one warp; every
+warp of the launch is placed once, those of shifted chunks first, each class
+spread evenly over its CTAs, also where a CTA holds both alignments; within a
+class the ranges (tests/c/split_ranges.h, the rule in its plain form) are
 cut by estimated segment cost (monotone boundaries covering every segment,
 the equal-count split for unit costs).  No GPU."""
 import os

@@ -2,16 +2,19 @@
 up to 2 of its lanes, lane by lane beyond that.
 
 A lane owns bytes 16l..16l+15 of every 512-byte block.  NaN and infinities put
-into 1 to 5 and 32 lanes of one segment take both ways, with elements whose
-squares under- or overflow fp32 among them (added in fp64) and in a segment cut
-short; counts must equal the oracle's and sums agree to 1e-9."""
+into 1 to 5 and 32 lanes of one segment take both ways, among ordinary values,
+in whole segments and short ones; so do lanes whose squares all underflow fp32
+and lanes with one that overflows it, each in a state of its own, so that every
+such square counts in the sum (added in fp64).  Counts must equal the oracle's
+and sums agree to 1e-9; and a lane's share must be the same bit for bit either
+way."""
 import os
 import subprocess
 
 import pytest
 import torch
 
-from gpu_helpers import compare_full
+from gpu_helpers import compare_full, table_np
 
 pytestmark = pytest.mark.gpu
 
@@ -19,27 +22,61 @@ fr = pytest.importorskip("paper_2509_03047_gb300.flashrec")
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
+def _rows(blocks, dtype, shift, base):
+    """A view of `base` off the 16-byte boundary by `shift` bytes, and the same as (block, lane, element of it)."""
+    n = blocks * 512 // dtype.itemsize
+    x = base[shift // dtype.itemsize:][:n]
+    return x, x.view(blocks, 32, 16 // dtype.itemsize)
+
+
 @pytest.mark.parametrize("shift", [0, 4])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("lanes", [1, 2, 3, 4, 5, 32])
-def test_segments_redone_exactly(dtype, lanes, shift):
+@pytest.mark.parametrize("kind", ["nan", "tiny", "huge"])
+def test_segments_redone_exactly(dtype, lanes, shift, kind):
     gen = torch.Generator(device="cuda").manual_seed(lanes)
-    per_lane = 16 // dtype.itemsize
     tensors = []
     for blocks in (1, 31, 32, 33, 70):
-        n = blocks * 512 // dtype.itemsize
-        base = torch.randn(n + 16, generator=gen, device="cuda").to(dtype)
-        x = base[shift // dtype.itemsize:][:n]
-        rows = x.view(blocks, 32, per_lane)
+        base = torch.randn(blocks * 512 // dtype.itemsize + 16, generator=gen, device="cuda").to(dtype)
         where = torch.randperm(32, generator=gen, device="cuda")[:lanes]
-        rows[blocks // 2, where, 1] = float("nan")
-        rows[0, where[:1], 0] = float("-inf")
-        if blocks > 31:  # odd elements in the same lanes
-            rows[3, where, 2] = 1e-25
-            rows[5, where, 3] = 1e25
-            rows[7, where, 0] = 3e-39
+        if kind == "tiny":  # the sum is that of squares below fp32's range, in these lanes; exact zeros elsewhere
+            values = (base.float() * 1e-25).to(dtype)
+            x, rows = _rows(blocks, dtype, shift, values)
+            keep = torch.zeros(32, dtype=torch.bool, device="cuda")
+            keep[where] = True
+            rows[:, ~keep] = 0
+            rows[blocks // 2, where, 3] = 3e-39  # (subnormal)
+        else:
+            x, rows = _rows(blocks, dtype, shift, base)
+            if kind == "huge":
+                rows[blocks // 3, where, 3] = 1e25
+            else:
+                rows[blocks // 2, where, 1] = float("nan")
+                rows[0, where[:1], 0] = float("-inf")
         tensors.append(x)
     compare_full(tensors, 64 * 1024)
+
+
+@pytest.mark.parametrize("shift", [0, 4])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_one_lane_adds_the_same_bits_with_others_redone_beside_it(dtype, shift):
+    """Lane 9 alone, and the same with lanes that hold NaN only, which add nothing but make the lanes go side by side."""
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    values = torch.randn(32, 16 // dtype.itemsize, generator=gen, device="cuda").to(dtype)
+    values[7, 1], values[8, 0], values[9, 2] = float("nan"), 1e-25, 1e-41
+    tensors = []
+    for others in (0, 1, 2, 4, 31):
+        x, rows = _rows(32, dtype, shift, torch.zeros(16384 // dtype.itemsize + 16, dtype=dtype, device="cuda"))
+        rows[:, 9] = values
+        for lane in [l for l in range(32) if l != 9][:others]:
+            rows[:, lane] = float("nan")
+        tensors.append(x)
+    table = table_np(fr.Plan(tensors, 16 * 1024).fingerprint())
+    per_lane = values.numel()
+    assert table["nonfinite"].tolist() == [1 + n * per_lane for n in (0, 1, 2, 4, 31)]
+    assert len(set(table["sumsq"].view("int64").tolist())) == 1
+    want = float(values.double().masked_fill(values.isnan(), 0.0).square().sum())
+    assert abs(table["sumsq"][0] - want) <= 1e-9 * want
 
 
 @pytest.mark.parametrize("seg_blocks", [32, 64])

@@ -2,7 +2,9 @@
 too early or written too late, whatever runs before and after on the stream:
 results of calls enqueued back to back, with other kernels rewriting their
 inputs in between, equal those of the same calls with a wait after each; and a
-pipeline over two streams replays from a graph."""
+pipeline over two streams replays from a graph.  Source and destination lie on
+and off the 16-byte boundary: the sweeps of shifted chunks keep what they read
+in L1."""
 import pytest
 import torch
 
@@ -11,22 +13,38 @@ pytestmark = pytest.mark.gpu
 fr = pytest.importorskip("paper_2509_03047_gb300.flashrec")
 
 
-def _state(sizes, seed=0):
+# (element type, bytes off the 16-byte boundary of the source, of the destination)
+PLACES = [(torch.float32, 0, 0), (torch.float32, 4, 0), (torch.float32, 0, 4), (torch.bfloat16, 2, 6)]
+
+
+def _views(sizes, dtype, shift):
+    """Zeros, each tensor `shift` bytes off the boundary."""
+    k = shift // dtype.itemsize
+    return [torch.zeros(n + k, dtype=dtype, device="cuda")[k:] for n in sizes]
+
+
+def _state(sizes, dtype, shift, seed=0):
     g = torch.Generator(device="cuda").manual_seed(seed)
-    return [torch.randn(n, device="cuda", generator=g) for n in sizes]
+    out = _views(sizes, dtype, shift)
+    for t in out:
+        t.copy_(torch.randn(t.numel(), device="cuda", generator=g))
+    return out
 
 
 def _sizes(total):
-    """fp32 tensors of odd sizes: one large, some with a tail, some of less than a block."""
+    """Tensors of odd sizes: one large, some with a tail, some of less than a block."""
     return [total, 1, 127, 128, 4099, 65536 + 3, 33, 262144 + 77]
 
 
 # chunk counts below and above one tile of the compaction, and a state of many waves of finalize
+@pytest.mark.parametrize("place", PLACES)
 @pytest.mark.parametrize("total,chunk", [(1000, 4096), (1 << 20, 16384), (40 << 20, 4096), (40 << 20, 1 << 20)])
-def test_back_to_back_calls_equal_calls_with_waits(total, chunk):
+def test_back_to_back_calls_equal_calls_with_waits(total, chunk, place):
+    dtype, shift, shift_out = place
+
     def run(wait):
-        src = _state(_sizes(total))
-        dst = [torch.zeros_like(t) for t in src]
+        src = _state(_sizes(total), dtype, shift)
+        dst = _views(_sizes(total), dtype, shift_out)
         a, b = fr.Plan(src, chunk), fr.Plan(dst, chunk)
         packed, out = a.new_packed(), []
         mism = torch.empty(a.n_chunks, dtype=torch.int32, device="cuda")
@@ -70,15 +88,16 @@ def test_back_to_back_calls_equal_calls_with_waits(total, chunk):
     assert all(torch.equal(x, y) for x, y in zip(got, want))
 
 
-def test_batches_on_two_streams_replay_from_a_graph():
-    src = _state(_sizes(8 << 20), 1)
-    dst = [torch.zeros_like(t) for t in src]
+@pytest.mark.parametrize("place", PLACES)
+def test_batches_on_two_streams_replay_from_a_graph(place):
+    dtype, shift, shift_out = place
+    src = _state(_sizes(8 << 20), dtype, shift, 1)
+    dst = _views(_sizes(8 << 20), dtype, shift_out)
     batches = 6
     a = fr.fr_plan_create_batched(src, 65536, batches)
     b = fr.fr_plan_create_batched(dst, 65536, batches)
     whole = fr.Plan(src, 65536)
     packed, want = whole.new_packed(), whole.new_packed()
-    fr.fr_pack(whole.handle, want)
     count = torch.empty(1, dtype=torch.int64, device="cuda")
     s, r = torch.cuda.Stream(), torch.cuda.Stream()
 
@@ -96,6 +115,9 @@ def test_batches_on_two_streams_replay_from_a_graph():
     with torch.cuda.graph(g, stream=s):
         pipeline()
     for k in range(3):
+        for t in src:
+            t.add_(1)
+        fr.fr_pack(whole.handle, want)
         for t in dst:
             t.fill_(k)
         packed.fill_(k)

@@ -214,7 +214,7 @@ __device__ __forceinline__ uint32_t mul_lane(uint32_t a, uint32_t lb) {
 
 // ------------------------------------------------------------------ memory
 
-// 16 bytes at p, a multiple of 16.
+// 16 bytes at p, a multiple of 16.  (Non-coherent: see wait_for_kernel_before.)
 __device__ __forceinline__ uint4 ld_unit(const uint8_t* p) {
   uint4 v;
   asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"

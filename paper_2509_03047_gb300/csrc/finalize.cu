@@ -155,7 +155,7 @@ __device__ __forceinline__ void two_sum_pair(float& hi, float& lo, float bh, flo
 __device__ __forceinline__ void tail_elem(uint32_t f, uint32_t& nf, float& hi, float& lo, bool& odd) {
   const bool nonfinite = (f & 0x7F800000u) == 0x7F800000u;
   const float ax = fabsf(__uint_as_float(f));
-  const bool fast = ax == 0.0f || (ax >= 0x1p-40f && ax <= 0x1p56f);  // false for NaN and Inf
+  const bool fast = ax == 0.0f || pair_square(ax);  // false for NaN and Inf
   nf += nonfinite ? 1u : 0u;
   odd |= !fast && !nonfinite;
   const float x = fast ? __uint_as_float(f) : 0.0f;
@@ -166,7 +166,7 @@ __device__ __forceinline__ void tail_elem(uint32_t f, uint32_t& nf, float& hi, f
 // The fp64 share of a tail element that tail_elem left out (0 for the rest).
 __device__ __forceinline__ double tail_elem_odd(uint32_t f) {
   const float ax = fabsf(__uint_as_float(f));
-  const bool fast = ax == 0.0f || (ax >= 0x1p-40f && ax <= 0x1p56f);
+  const bool fast = ax == 0.0f || pair_square(ax);
   if (fast || (f & 0x7F800000u) == 0x7F800000u) return 0.0;
   const double d = static_cast<double>(__uint_as_float(f));
   return __dmul_rn(d, d);

@@ -115,6 +115,13 @@ __device__ __forceinline__ void wait_for_kernel_before() { asm volatile("griddep
 // wait_for_kernel_before, so that the next kernel starts after all that came
 // before this one.)
 __device__ __forceinline__ void allow_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// The one rule, in the sweeps' exact fallback and in finalize's tails, by which
+// the square of a finite element is added exactly to a float pair: |x| = ax in
+// [2^-40, 2^56], where the fp32 product and its FMA residual are the square (the
+// residual is not subnormal) and a lane's squares stay far from overflow.  A
+// zero adds nothing; any other square is added in fp64.
+__device__ __forceinline__ bool pair_square(float ax) { return ax >= 0x1p-40f && ax <= 0x1p56f; }
 #endif
 
 // Per device, before the first launch: opt the sweep kernels in to their

@@ -385,11 +385,21 @@ struct Exact {
 };
 
 
+// (hi, lo) += x * x exactly, for pair_square(|x|) or x = 0: the fp32 product and
+// its FMA residual, by TwoSum.
+__device__ __forceinline__ void add_pair_square(float& hi, float& lo, float x) {
+  const float p = x * x;
+  const float e = __fmaf_rn(x, x, -p);
+  const float t = hi + p;
+  const float z = t - hi;
+  lo += ((hi - (t - z)) + (p - z)) + e;
+  hi = t;
+}
+
 // Exact sum of squares of elements added one by one, in order, given as fp32
 // bit patterns (a bf16 element in the high half).  A non-finite element is
-// counted; the square of one with |x| = 0 or in [2^-40, 2^56] is added exactly
-// -- the fp32 product and its FMA residual -- to the float pair (hi, lo) by
-// TwoSum; any other sets `odd`, and odd_squares adds it.  No branch and no fp64
+// counted; a square that pair_square takes is added to the float pair (hi, lo);
+// any other sets `odd`, and odd_squares adds it.  No branch and no fp64
 // instruction: predicated off, those still take turns on the narrow pipe, and
 // with them in the loop a NaN cost the launch 13 us, without 2.
 struct ExactSum {
@@ -399,16 +409,10 @@ struct ExactSum {
   __device__ __forceinline__ void add(uint32_t f) {
     const bool inf_nan = (f & 0x7F800000u) == 0x7F800000u;
     const float ax = fabsf(__uint_as_float(f));
-    const bool fast = ax == 0.0f || (ax >= 0x1p-40f && ax <= 0x1p56f);  // false for NaN and Inf
+    const bool fast = ax == 0.0f || pair_square(ax);  // false for NaN and Inf
     nonfinite += inf_nan ? 1u : 0u;
     odd |= !fast && !inf_nan;
-    const float x = fast ? __uint_as_float(f) : 0.0f;  // (a zero square changes nothing)
-    const float p = x * x;
-    const float e = __fmaf_rn(x, x, -p);
-    const float t = hi + p;
-    const float z = t - hi;
-    lo += ((hi - (t - z)) + (p - z)) + e;
-    hi = t;
+    add_pair_square(hi, lo, fast ? __uint_as_float(f) : 0.0f);  // (a zero square changes nothing)
   }
   template <int DT>
   __device__ __forceinline__ void add_word(uint32_t w) {
@@ -431,7 +435,7 @@ __device__ __noinline__ double odd_squares(const uint8_t* sp, uint32_t n) {
     for (int j = 0; j < (DT == kDtF32 ? 4 : 8); ++j) {
       const uint32_t f = DT == kDtF32 ? w[j & 3] : ((j & 1) ? w[j / 2] & 0xFFFF0000u : w[j / 2] << 16);
       const float ax = fabsf(__uint_as_float(f));
-      if ((f & 0x7F800000u) == 0x7F800000u || ax == 0.0f || (ax >= 0x1p-40f && ax <= 0x1p56f)) continue;
+      if ((f & 0x7F800000u) == 0x7F800000u || ax == 0.0f || pair_square(ax)) continue;
       const double xd = static_cast<double>(__uint_as_float(f));
       d = __dadd_rn(d, __dmul_rn(xd, xd));
     }
@@ -470,13 +474,8 @@ __device__ __noinline__ Exact slow_span(const uint8_t* sp, uint32_t n) {
         }
         const float x = __uint_as_float(f);
         const float ax = fabsf(x);
-        if (ax >= 0x1p-40f && ax <= 0x1p56f) {
-          const float p2 = x * x;
-          const float e = __fmaf_rn(x, x, -p2);
-          const float t = hi + p2;
-          const float z = t - hi;
-          lo += ((hi - (t - z)) + (p2 - z)) + e;
-          hi = t;
+        if (pair_square(ax)) {
+          add_pair_square(hi, lo, x);
         } else if (ax != 0.0f) {
           const double xd = static_cast<double>(x);
           d = __dadd_rn(d, __dmul_rn(xd, xd));

@@ -930,13 +930,16 @@ fr_status fr_sync_status(fr_plan p, void* stream) {
   if (p == nullptr) return invalid("plan is null");
   DeviceGuard g(p->device);
   if (!g.ok) return cuda_fail(cudaGetLastError(), "select plan device");
-  cudaError_t e = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
+  const cudaStream_t s = static_cast<cudaStream_t>(stream);
+  cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
   uint32_t bits = 0;
   e = cudaMemcpy(&bits, p->d_status, sizeof bits, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "read plan status");
   if (bits == 0) return FR_OK;
-  e = cudaMemset(p->d_status, 0, sizeof bits);
+  // (waited for: the next call may be on any stream)
+  e = cudaMemsetAsync(p->d_status, 0, sizeof bits, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "clear plan status");
   if (bits & kStatusTimeout) return FR_ERR_DEVICE_TIMEOUT;
   return FR_ERR_CAPACITY;

@@ -76,7 +76,9 @@ constexpr int kTableBytes = 4 * 256 * 32 * 4;  // 4 tables x 256 entries x 32 la
 // same together however many.  Measured, fingerprint of 15 MB of fp32 as a
 // graph, us, in turn / side by side, NaN lanes in one segment: 1 lane 17 / 25, 2
 // lanes 20 / 25, 3 lanes 24 / 25, 4 lanes 27 / 25; in every segment: 22 / 27, 30 /
-// 27, 37 / 27, 44 / 27.
+// 27, 37 / 27, 44 / 27.  Among lanes whose squares are tiny (span_end_slow) only
+// one is taken so: their squares are added one by one in fp64 (256 MB of
+// exp(N(ln 1e-12, 3^2)): fingerprint, up to 1 / 2 lanes in turn, 409 / 426).
 #ifndef FR_SLOW_WARP_LANES
 #define FR_SLOW_WARP_LANES 2
 #endif
@@ -399,7 +401,7 @@ __device__ __forceinline__ void add_pair_square(float& hi, float& lo, float x) {
 // Exact sum of squares of elements added one by one, in order, given as fp32
 // bit patterns (a bf16 element in the high half).  A non-finite element is
 // counted; a square that pair_square takes is added to the float pair (hi, lo);
-// any other sets `odd`, and odd_squares adds it.  No branch and no fp64
+// any other sets `odd`, and the caller adds it (odd_elem).  No branch and no fp64
 // instruction: predicated off, those still take turns on the narrow pipe, and
 // with them in the loop a NaN cost the launch 13 us, without 2.
 struct ExactSum {
@@ -421,26 +423,26 @@ struct ExactSum {
   }
 };
 
-// The squares that ExactSum leaves out (tiny or huge values, rare), of the
-// calling lane's units of `n` blocks, the first at sp, in order: in fp64, where
-// the square of an fp32 value is exact.
-template <int DT, bool SHIFT>
-__device__ __noinline__ double odd_squares(const uint8_t* sp, uint32_t n) {
-  double d = 0.0;
-#pragma unroll 1
-  for (uint32_t b = 0; b < n; ++b) {
-    const uint4 v = ld_unit_at<SHIFT>(sp + b * kBlockBytes);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+// Whether an element, given as fp32 bits, has a square that ExactSum leaves out
+// (tiny or huge, rare), and the sum of those of a word, in fp64, where the
+// square of an fp32 value is exact.
+__device__ __forceinline__ bool odd_elem(uint32_t f) {
+  const float ax = fabsf(__uint_as_float(f));
+  return (f & 0x7F800000u) != 0x7F800000u && ax != 0.0f && !pair_square(ax);
+}
+template <int DT>
+__device__ __forceinline__ bool odd_word(uint32_t w) {
+  return DT == kDtF32 ? odd_elem(w) : odd_elem(w << 16) || odd_elem(w & 0xFFFF0000u);
+}
+template <int DT>
+__device__ __forceinline__ void add_odd(double& d, uint32_t w) {
 #pragma unroll
-    for (int j = 0; j < (DT == kDtF32 ? 4 : 8); ++j) {
-      const uint32_t f = DT == kDtF32 ? w[j & 3] : ((j & 1) ? w[j / 2] & 0xFFFF0000u : w[j / 2] << 16);
-      const float ax = fabsf(__uint_as_float(f));
-      if ((f & 0x7F800000u) == 0x7F800000u || ax == 0.0f || pair_square(ax)) continue;
-      const double xd = static_cast<double>(__uint_as_float(f));
-      d = __dadd_rn(d, __dmul_rn(xd, xd));
-    }
+  for (int h = 0; h < (DT == kDtF32 ? 1 : 2); ++h) {
+    const uint32_t f = DT == kDtF32 ? w : h == 0 ? w << 16 : w & 0xFFFF0000u;
+    if (!odd_elem(f)) continue;
+    const double xd = static_cast<double>(__uint_as_float(f));
+    d = __dadd_rn(d, __dmul_rn(xd, xd));
   }
-  return d;
 }
 
 // Exact per-element fallback for this lane's units of `n` blocks, the first at sp:
@@ -497,6 +499,7 @@ template <int DT, bool SHIFT>
 __device__ __noinline__ Exact slow_span_by_warp(const uint8_t* sp, uint32_t n, uint32_t l, uint32_t lane) {
   const uint8_t* first = sp + (static_cast<int32_t>(l) - static_cast<int32_t>(lane)) * 16;  // lane l's first unit
   ExactSum x;
+  double d = 0.0;  // the squares that x leaves out, in the same order
 #pragma unroll 1
   for (uint32_t g = 0; g < kSpan; g += 32) {  // (one pass unless a segment is built larger)
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -508,8 +511,23 @@ __device__ __noinline__ Exact slow_span_by_warp(const uint8_t* sp, uint32_t n, u
       x.add_word<DT>(__shfl_sync(0xFFFFFFFFu, v.z, k - g));
       x.add_word<DT>(__shfl_sync(0xFFFFFFFFu, v.w, k - g));
     }
+    if (x.odd) {
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+      uint32_t odd = 0;  // the words of this lane's unit that hold one
+#pragma unroll
+      for (int j = 0; j < 4; ++j) odd |= (odd_word<DT>(w[j]) ? 1u : 0u) << j;
+#pragma unroll 1
+      for (uint32_t m = __ballot_sync(0xFFFFFFFFu, odd != 0); m != 0; m &= m - 1) {
+        const int k = __ffs(static_cast<int>(m)) - 1;
+        const uint32_t o = __shfl_sync(0xFFFFFFFFu, odd, k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t wj = __shfl_sync(0xFFFFFFFFu, w[j], k);
+          if (o >> j & 1u) add_odd<DT>(d, wj);
+        }
+      }
+    }
   }
-  const double d = x.odd ? odd_squares<DT, SHIFT>(first, n) : 0.0;
   return Exact{(static_cast<double>(x.hi) + static_cast<double>(x.lo)) + d, x.nonfinite};
 }
 
@@ -644,7 +662,8 @@ __device__ __noinline__ uint32_t span_end_slow(FpAcc f, float tot, const uint8_t
   }
   if (ok) d = static_cast<double>(hi) + static_cast<double>(lo);
   uint32_t bad = __ballot_sync(0xFFFFFFFFu, !ok);
-  if (__popc(bad) > kSlowWarpLanes) {
+  const bool tiny = __any_sync(0xFFFFFFFFu, !ok && tot < 1.0f);  // (else NaN, Inf or overflow)
+  if (__popc(bad) > (tiny ? 1 : kSlowWarpLanes)) {
     bad = 0;
     if (!ok) {
       const Exact x = slow_span<DT, SHIFT>(sp, n);

@@ -1,5 +1,5 @@
 """GPU tests of the sum segments that are redone exactly: by the whole warp for
-up to 2 of its lanes, lane by lane beyond that.
+up to 2 of its lanes (1 where squares are tiny), lane by lane beyond that.
 
 A lane owns bytes 16l..16l+15 of every 512-byte block.  NaN and infinities put
 into 1 to 5 and 32 lanes of one segment take both ways, among ordinary values,
@@ -55,6 +55,18 @@ def test_segments_redone_exactly(dtype, lanes, shift, kind):
                 rows[0, where[:1], 0] = float("-inf")
         tensors.append(x)
     compare_full(tensors, 64 * 1024)
+
+
+@pytest.mark.parametrize("shift", [0, 4])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("center", [1e-12, 1e-11, 1e-10])
+def test_second_moments_around_the_line(dtype, center, shift):
+    """Values spread as Adam's second moments are: from none to all lanes of a segment have sums too small for the fast
+    path, with elements among them whose squares are added in fp64."""
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    n = 60 * 16384 // dtype.itemsize
+    values = torch.randn(n + 16, generator=gen, device="cuda").mul_(2.0).exp_().mul_(center).to(dtype)
+    compare_full([values[shift // dtype.itemsize:][:n]], 64 * 1024)
 
 
 @pytest.mark.parametrize("shift", [0, 4])

@@ -269,8 +269,10 @@ void build_decomp(const std::vector<ChunkDesc>& base, const std::vector<uint64_t
     double cost[kClassCount];
     uint64_t wc[kClassCount];
     int n_cls = 0;
+    bool shifted = false, aligned = false;
     for (uint32_t cls = 0; cls < kClassCount; ++cls) {
       if (blocks[cls] == 0) continue;
+      (cls & 1u ? aligned : shifted) = true;
       cls_of[n_cls] = cls;
       cost[n_cls++] = static_cast<double>(blocks[cls]) * class_weight(cls, share);
     }
@@ -283,7 +285,7 @@ void build_decomp(const std::vector<ChunkDesc>& base, const std::vector<uint64_t
     for (int q = 0; q < n_cls; ++q) {
       const uint32_t cls = cls_of[q];
       const uint64_t n_seg = segs[cls], Wq = wc[q];
-      const uint64_t n_fix = n_seg - claimed_segs(n_seg, Wq, share);  // segments in the warps' runs
+      const uint64_t n_fix = n_seg - claimed_segs(n_seg, Wq, share, cls, shifted && aligned);  // in the warps' runs
       SegWalk at(chunks.data(), lists[cls].data(), lists[cls].size());
       SegWalk fixed = at;
       fixed.skip(n_fix);

@@ -64,6 +64,17 @@
 #ifndef FR_DYN_PCT
 #define FR_DYN_PCT 8
 #endif
+// The classes of shifted chunks keep FR_DYN_PCT_MIXED percent in a launch that
+// holds aligned classes too.  They have SMs of their own (place_warps), on which
+// a block of unpack takes longer, and pack and unpack share one plan, so no
+// weight suits both (10% more warps for them: unpack 351 -> 337 us below, but
+// flat views' pack 777 -> 811).  Measured with 8 / 12 / 16 / 24 percent, 1 GB in
+// eight fp32 tensors, one of them shifted: unpack 350 / 342 / 335 / 331 us, pack
+// 333 either way; 2.5 GB of flat views, pack and unpack with both tables: 1,585 /
+// 1,592 / 1,588 / 1,593.  Where every class is shifted 16 percent cost unpack 1%.
+#ifndef FR_DYN_PCT_MIXED
+#define FR_DYN_PCT_MIXED 16
+#endif
 #ifndef FR_UNIT_SEGS
 #define FR_UNIT_SEGS 2
 #endif
@@ -140,11 +151,13 @@ inline uint64_t seg_cost(uint64_t blocks, bool first) {
   return FR_SPLIT_BLK * blocks + FR_SPLIT_SEG + (first ? FR_SPLIT_PIECE : 0);
 }
 
-// How many of the last segments of a class of n, shared by Wq warps, are cut
-// into units (none for the fingerprint, see mode_claims, nor while the warps
-// have too few segments each for a tail to even out).
-inline uint64_t claimed_segs(uint64_t n, uint64_t Wq, int kind) {
-  return kind == kShareFingerprint || n < FR_CLAIM_MIN * Wq ? 0 : n * FR_DYN_PCT / 100;
+// How many of the last segments of sweep class `cls`, of n in all and shared by
+// Wq warps, are cut into units (none for the fingerprint, see mode_claims, nor
+// while the warps have too few segments each for a tail to even out).  `mixed`:
+// the launch holds classes of both alignments.
+inline uint64_t claimed_segs(uint64_t n, uint64_t Wq, int kind, uint32_t cls, bool mixed) {
+  const uint64_t percent = mixed && (cls & 1u) == 0 ? FR_DYN_PCT_MIXED : FR_DYN_PCT;
+  return kind == kShareFingerprint || n < FR_CLAIM_MIN * Wq ? 0 : n * percent / 100;
 }
 // Segments of the unit cut where `left` remain: a share of what is left, so
 // that a large state has few units and a chunk of it few records, down to

@@ -78,9 +78,14 @@ __host__ __device__ constexpr int sweep_warps(int mode) {
 // for it, and with it for all before it, before it touches memory that any
 // kernel writes.  A kernel of someone else's in between is waited for whole.
 // GB300, us, launched one after the other -> so: GPT-2 small fingerprint 280 ->
-// 276 (277 without allow_next_kernel), pack 539 -> 534, unpack 538 -> 532; 4.2
-// GB in 50,000 tensors, fingerprint 677 -> 672; GPT-2 small restored in 16
-// batches 1540 -> 1465; a 15 MB state's restore step 39.3 -> 37.4.
+// 276, pack 539 -> 534, unpack 538 -> 532; 4.2 GB in 50,000 tensors, fingerprint
+// 677 -> 672; GPT-2 small restored in 16 batches 1540 -> 1465; a 15 MB state's
+// restore step 39.3 -> 37.4.  No kernel lets the next start before its own blocks
+// end (griddepcontrol.launch_dependents): finalize's blocks on the SMs that finish
+// first slow the sweep's last ones.  With the trigger / without, us: fingerprint
+// of 64 MB 22.7 / 20.1, 256 MB 57.9 / 57.1, 1 GB 178 / 175, 1.7 GB and more equal
+// (a mix of bf16 and fp32 of 320 to 400 MB 1 us less with it); pack and unpack of
+// GPT-2 small in 16 batches 1547 / 1461.
 template <class... P>
 cudaError_t launch_chained(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, const P&... args) {
   cudaLaunchAttribute overlap = {};
@@ -110,11 +115,6 @@ cudaError_t launch_chained(void (*kernel)(P...), int grid, int block, size_t sme
 // before them: 2.5 GB of views, pack 781 -> 944 us, unpack 788 -> 1,003; aligned
 // states equal but for the Llama-8B step, 8,377 -> 8,399.
 __device__ __forceinline__ void wait_for_kernel_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// From here on blocks of the next kernel may take the place of this one's
-// finished blocks, not only once all are finished.  (Called after
-// wait_for_kernel_before, so that the next kernel starts after all that came
-// before this one.)
-__device__ __forceinline__ void allow_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // The one rule, in the sweeps' exact fallback and in finalize's tails, by which
 // the square of a finite element is added exactly to a float pair: |x| = ax in

@@ -940,11 +940,6 @@ template <int MODE>
 __global__ void __launch_bounds__(Cta<MODE>::kThreads, 1) sweep_kernel(SweepParams p) {
   fill_smem<MODE>();
   wait_for_kernel_before();
-  // Finalize's blocks may settle on the SMs that finish first.  Pack and unpack
-  // lose by it: their batches share the SMs with another stream's sweep, which
-  // then finds them taken (GPT-2 small in 16 batches 1461 -> 1547 us, the 15 MB
-  // state's step 37.0 -> 39.8).
-  if (MODE == kModeFingerprint) allow_next_kernel();
   const uint32_t lane = threadIdx.x & 31u;
   RunDesc rd = p.warps[blockIdx.x * Cta<MODE>::kWarps + (threadIdx.x >> 5)];
   for (;;) {

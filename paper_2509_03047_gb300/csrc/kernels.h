@@ -83,9 +83,9 @@ __host__ __device__ constexpr int sweep_warps(int mode) {
 // restore step 39.3 -> 37.4.  No kernel lets the next start before its own blocks
 // end (griddepcontrol.launch_dependents): finalize's blocks on the SMs that finish
 // first slow the sweep's last ones.  With the trigger / without, us: fingerprint
-// of 64 MB 22.7 / 20.1, 256 MB 57.9 / 57.1, 1 GB 178 / 175, 1.7 GB and more equal
-// (a mix of bf16 and fp32 of 320 to 400 MB 1 us less with it); pack and unpack of
-// GPT-2 small in 16 batches 1547 / 1461.
+// of 64 MB 22.7 / 20.1, 256 MB 57.9 / 57.1, 1 GB 178 / 175, 1.7 to 14 GB equal,
+// 32 GB in 16 MiB chunks 4,935 / 4,945 (a mix of bf16 and fp32 of 320 to 400 MB 1
+// us less with it); pack and unpack of GPT-2 small in 16 batches 1547 / 1461.
 template <class... P>
 cudaError_t launch_chained(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, const P&... args) {
   cudaLaunchAttribute overlap = {};
